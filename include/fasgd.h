@@ -369,9 +369,9 @@ FASGD_API int bfasgd_fetch_budget(fasgd_t* h, int32_t client, float* theta_clien
  * fasgd_pull -- copy theta (P fp32) into params (host or device) and return
  * the server timestamp T in *T (Sec. 2.1 protocol step 3: the parameters
  * handed back to a client).  The copy is ordered after earlier work on the
- * handle's stream and later work on that stream waits for it (it runs on an
- * internal stream beside pending host-push copies).  Pending pushes are not
- * applied.
+ * handle's stream and later work on that stream waits for it (a copy to host
+ * memory runs on an internal stream beside pending host-push copies).
+ * Pending pushes are not applied.
  * Either output may be NULL.  Errors: EINVAL, ECUDA.
  */
 FASGD_API int fasgd_pull(fasgd_t* h, float* params, int64_t* T);
@@ -428,7 +428,9 @@ FASGD_API int fasgd_selftest_fail_pass(fasgd_t* h, int32_t after);
 FASGD_API int64_t fasgd_timestamp(const fasgd_t* h);
 FASGD_API int64_t fasgd_pending(const fasgd_t* h);
 
-/* Number of kernels this handle has launched since it was created. */
+/* Number of kernels of the update and B-FASGD paths this handle has launched
+ * since it was created (the copies of fasgd_pull and fasgd_get_state are not
+ * counted). */
 FASGD_API int64_t fasgd_kernel_launches(const fasgd_t* h);
 
 /*

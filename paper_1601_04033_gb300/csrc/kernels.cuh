@@ -109,6 +109,15 @@ struct ScatterArgs {
     int32_t* err;              // may be null; flags 1 (count) and 2 (index)
 };
 
+// Copies of up to four of the server's arrays (copy.cu): dst[i] <- src[i],
+// P floats each; src 16-byte aligned, dst 4-byte aligned device memory.
+struct CopyArgs {
+    const float* src[4];
+    float* dst[4];
+    int32_t count;
+    int64_t P;
+};
+
 // Closed-loop simulation: stochastic gradient and loss of the synthetic
 // quadratic objective (sim.cu).
 struct SimGradArgs {
@@ -141,6 +150,7 @@ cudaError_t launch_dense(const DenseArgs& a, int rule, bool exact, int num_sms, 
 cudaError_t launch_sparse(const SparseArgs& a, int rule, bool exact, int num_sms, cudaStream_t stream,
                           int64_t* launches);
 cudaError_t launch_select(const SelectArgs& a, cudaStream_t stream, int64_t* launches);
+cudaError_t launch_copy(const CopyArgs& a, int num_sms, cudaStream_t stream);
 cudaError_t launch_scatter(const ScatterArgs& a, int num_sms, cudaStream_t stream);
 // Self-test: bounded pipeline waits that can never complete (raise flag 8 in err).
 cudaError_t launch_wait_expiry(int32_t* err, cudaStream_t stream);

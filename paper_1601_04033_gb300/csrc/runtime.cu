@@ -71,6 +71,18 @@ std::string vformat(const char* fmt, va_list ap) {
     return buf;
 }
 
+// Whether p can be written by a copy kernel on `device`: device memory of that
+// device (not host, managed or a peer's memory), aligned to a float.
+bool local_device_floats(const void* p, int device) {
+    if (!aligned(p, 4)) return false;
+    cudaPointerAttributes attr;
+    if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
+        cudaGetLastError();   // an unknown pointer is left to cudaMemcpyAsync
+        return false;
+    }
+    return attr.type == cudaMemoryTypeDevice && attr.device == device;
+}
+
 // Makes h's device current for the lifetime of the guard.
 struct DeviceGuard {
     int prev = -1;
@@ -1112,11 +1124,25 @@ int fasgd_pull(fasgd_t* h, float* params, int64_t* T) {
     TraceRange trace("fasgd_pull");
     if (h == nullptr) return FASGD_EINVAL;
     if (params != nullptr) {
-        // The copy runs on its own stream (so it overlaps host-push copies of
-        // the next pushes) and the handle's stream waits for it: later work on
-        // the stream, and a caller synchronising it, see the pull complete.
         DeviceGuard g(h->device);
-        cudaError_t st = h->ensure_aux();
+        cudaError_t st = cudaSuccess;
+        if (local_device_floats(params, h->device)) {
+            // Device memory: one kernel on the handle's stream, in order.
+            fasgd::CopyArgs c;
+            std::memset(&c, 0, sizeof c);
+            c.src[0] = h->theta;
+            c.dst[0] = params;
+            c.count = 1;
+            c.P = h->P;
+            st = fasgd::launch_copy(c, h->num_sms, h->stream);
+            if (st != cudaSuccess) return h->cuda_fail(st, "fasgd_pull");
+            if (T != nullptr) *T = h->T;
+            return FASGD_OK;
+        }
+        // Host memory: the copy runs on its own stream (so it overlaps host-push
+        // copies of the next pushes) and the handle's stream waits for it: later
+        // work on the stream, and a caller synchronising it, see the pull complete.
+        st = h->ensure_aux();
         if (st == cudaSuccess) st = cudaEventRecord(h->order_ev, h->stream);
         if (st == cudaSuccess) st = cudaStreamWaitEvent(h->pull_stream, h->order_ev, 0);
         if (st == cudaSuccess)
@@ -1137,13 +1163,24 @@ int fasgd_get_state(fasgd_t* h, float* theta, float* n, float* b, float* v, int6
     DeviceGuard g(h->device);
     float* dst[] = {theta, n, b, v};
     const float* src[] = {h->theta, h->n, h->b, h->v};
-    for (int i = 0; i < 4; ++i) {
+    // Arrays wanted in device memory go in one kernel, the others by copies.
+    fasgd::CopyArgs c;
+    std::memset(&c, 0, sizeof c);
+    c.P = h->P;
+    cudaError_t st = cudaSuccess;
+    for (int i = 0; i < 4 && st == cudaSuccess; ++i) {
         if (dst[i] == nullptr) continue;
-        cudaError_t st = cudaMemcpyAsync(dst[i], src[i], (size_t)h->P * sizeof(float),
-                                         cudaMemcpyDefault, h->stream);
-        if (st != cudaSuccess) return h->cuda_fail(st, "fasgd_get_state");
+        if (local_device_floats(dst[i], h->device)) {
+            c.src[c.count] = src[i];
+            c.dst[c.count++] = dst[i];
+        } else {
+            st = cudaMemcpyAsync(dst[i], src[i], (size_t)h->P * sizeof(float), cudaMemcpyDefault,
+                                 h->stream);
+        }
     }
-    cudaError_t st = cudaStreamSynchronize(h->stream);
+    if (st == cudaSuccess && c.count > 0) st = fasgd::launch_copy(c, h->num_sms, h->stream);
+    if (st != cudaSuccess) return h->cuda_fail(st, "fasgd_get_state");
+    st = cudaStreamSynchronize(h->stream);
     if (st != cudaSuccess) return h->cuda_fail(st, "fasgd_get_state");
     if (T != nullptr) *T = h->T;
     return FASGD_OK;
