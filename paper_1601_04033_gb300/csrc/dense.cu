@@ -75,22 +75,15 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
         : "memory");
 }
 
-// ---- the element update on four consecutive parameters --------------------
-template <int RULE, int ARITH>
-__device__ __forceinline__ void update4(float4& th, float4& n, float4& b, float4& v, const float4& g,
-                                        float coef, const StatParams& sp) {
-    constexpr bool STD = RULE == kRuleFasgdStd;
-    if (RULE != kRuleSgd) {
-        rule_update<ARITH, STD>(th.x, n.x, b.x, v.x, g.x, coef, sp);
-        rule_update<ARITH, STD>(th.y, n.y, b.y, v.y, g.y, coef, sp);
-        rule_update<ARITH, STD>(th.z, n.z, b.z, v.z, g.z, coef, sp);
-        rule_update<ARITH, STD>(th.w, n.w, b.w, v.w, g.w, coef, sp);
-    } else {
-        sgd_update(th.x, g.x, coef);
-        sgd_update(th.y, g.y, coef);
-        sgd_update(th.z, g.z, coef);
-        sgd_update(th.w, g.w, coef);
-    }
+// A quad whose exact arithmetic left the range of its fast form.
+template <int RULE>
+__device__ __forceinline__ void redo_quad(const DenseArgs& a, const float* g0, int64_t e, float4& th,
+                                          float4& n, float4& b, float4& v) {
+    const QuadState q = exact_quad<RULE == kRuleFasgdStd>(a.theta, a.n, a.b, a.v, g0, a.grad, a.coef, a.K, e, a.sp);
+    th = q.th;
+    n = q.n;
+    b = q.b;
+    v = q.v;
 }
 
 // Parameters [begin, P) with plain loads, by the CONS consumer threads of
@@ -107,10 +100,12 @@ __device__ void apply_range_direct(const DenseArgs& a, int64_t begin, int tid) {
             b = *reinterpret_cast<const float4*>(a.b + e);
             v = *reinterpret_cast<const float4*>(a.v + e);
         }
+        Guard<ARITH> guard;
         for (int k = 0; k < a.K; ++k) {
             const float4 g = __ldcs(reinterpret_cast<const float4*>(a.grad[k] + e));
-            update4<RULE, ARITH>(th, n, b, v, g, a.coef[k], a.sp);
+            update4<RULE, ARITH>(th, n, b, v, g, a.coef[k], a.sp, guard);
         }
+        if (!guard.ok()) redo_quad<RULE>(a, a.grad[0], e, th, n, b, v);
         *reinterpret_cast<float4*>(a.theta + e) = th;
         if (FAS) {
             *reinterpret_cast<float4*>(a.n + e) = n;
@@ -299,6 +294,7 @@ fasgd_dense_kernel(const __grid_constant__ DenseArgs a, const Ring ring, const i
     bool ok = true;
     for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         float4 th = make_float4(0.f, 0.f, 0.f, 0.f), n = th, b = th, v = th;
+        Guard<ARITH> guard;
         for (int c = 0; c < ring.chunks; ++c) {
             ok = wait_warp(&full[s], ph, a.err);
             if (!ok) break;
@@ -322,7 +318,7 @@ fasgd_dense_kernel(const __grid_constant__ DenseArgs a, const Ring ring, const i
                 if (SUMS && copy_to != nullptr)          // a transmitted message refreshes its slot
                     reinterpret_cast<float4*>(copy_to + t * kTile)[tid] = g[0];
 #pragma unroll
-                for (int j = 0; j < CH; ++j) update4<RULE, ARITH>(th, n, b, v, g[j], a.coef[k0 + j], a.sp);
+                for (int j = 0; j < CH; ++j) update4<RULE, ARITH>(th, n, b, v, g[j], a.coef[k0 + j], a.sp, guard);
             } else {               // the last, partial chunk
                 const int ng = a.K - k0;
 #pragma unroll
@@ -332,7 +328,7 @@ fasgd_dense_kernel(const __grid_constant__ DenseArgs a, const Ring ring, const i
                 if (lane == 0) mbar_arrive(&empty[s]);
 #pragma unroll
                 for (int j = 0; j < CH; ++j)
-                    if (j < ng) update4<RULE, ARITH>(th, n, b, v, g[j], a.coef[k0 + j], a.sp);
+                    if (j < ng) update4<RULE, ARITH>(th, n, b, v, g[j], a.coef[k0 + j], a.sp, guard);
             }
             if (++s == ring.stages) {
                 s = 0;
@@ -341,6 +337,7 @@ fasgd_dense_kernel(const __grid_constant__ DenseArgs a, const Ring ring, const i
         }
         if (!ok) break;
         const int64_t e = t * kTile + 4 * (int64_t)tid;
+        if (!guard.ok()) redo_quad<RULE>(a, g0, e, th, n, b, v);
         *reinterpret_cast<float4*>(a.theta + e) = th;
         if (FAS) {
             *reinterpret_cast<float4*>(a.n + e) = n;
@@ -426,6 +423,7 @@ fasgd_direct_kernel(const __grid_constant__ DenseArgs a) {
                 b = *reinterpret_cast<const float4*>(a.b + e);
                 v = *reinterpret_cast<const float4*>(a.v + e);
             }
+            Guard<ARITH> guard;
             for (int k0 = 0; k0 < a.K; k0 += 8) {
                 float4 g[8];
 #pragma unroll
@@ -433,8 +431,9 @@ fasgd_direct_kernel(const __grid_constant__ DenseArgs a) {
                     if (k0 + j < a.K) g[j] = *reinterpret_cast<const float4*>(a.grad[k0 + j] + e);
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
-                    if (k0 + j < a.K) update4<RULE, ARITH>(th, n, b, v, g[j], a.coef[k0 + j], a.sp);
+                    if (k0 + j < a.K) update4<RULE, ARITH>(th, n, b, v, g[j], a.coef[k0 + j], a.sp, guard);
             }
+            if (!guard.ok()) redo_quad<RULE>(a, a.grad[0], e, th, n, b, v);
             *reinterpret_cast<float4*>(a.theta + e) = th;
             if (FAS) {
                 *reinterpret_cast<float4*>(a.n + e) = n;
@@ -488,6 +487,10 @@ cudaError_t launch_rule(const DenseArgs& a, int num_sms, cudaStream_t stream) {
     // keep more stages in flight there (P = 50M, K = 16: 686.8 against
     // 704.0 us per pass); up to K = 8 one block of 512 is faster (226.8
     // against 232.1 us at P = 25M, K = 8).
+    // The exact rules hold more values per push: four slices at a time leave
+    // them the registers (K = 8 / 16 at 25M: 282 / 519 against 289 / 549 us
+    // with eight, push + apply + pull).
+    if (ARITH == kArithExact && RULE != kRuleSgd && a.K > 4) return launch_ch<RULE, ARITH, 4>(a, num_sms, stream);
     if (a.K > 8) return launch_ch<RULE, ARITH, 8, false, 256>(a, num_sms, stream);
     if (a.K > 4) return launch_ch<RULE, ARITH, 8>(a, num_sms, stream);
     if (a.K > 2) return launch_ch<RULE, ARITH, 4>(a, num_sms, stream);

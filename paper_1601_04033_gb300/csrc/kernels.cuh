@@ -20,6 +20,7 @@ struct StatParams {
     float gamma, one_m_gamma;
     float beta, one_m_beta;
     float eps;
+    float minus_zero;   // -0.0f, a value the compiler does not see (update.cuh, product2)
 };
 
 // A per-message push decided inside its pass (with vsum, FASGD rules): the

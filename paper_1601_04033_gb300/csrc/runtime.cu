@@ -355,6 +355,7 @@ struct fasgd_s {
         sp.beta = beta;
         sp.one_m_beta = 1.0f - beta;
         sp.eps = eps;
+        sp.minus_zero = -0.0f;
         return sp;
     }
     // alpha(tau) of Eq. 1 / Eq. 7 (the v factor of Eq. 7 is per element).

@@ -388,23 +388,6 @@ __global__ void __launch_bounds__(kTensorResolveThreads) budget_resolve_kernel(c
 }
 
 template <int RULE, int ARITH>
-__device__ __forceinline__ void update4(float4& th, float4& n, float4& b, float4& v, const float4& g,
-                                        float coef, const StatParams& sp) {
-    if (RULE == kRuleSgd) {
-        sgd_update(th.x, g.x, coef);
-        sgd_update(th.y, g.y, coef);
-        sgd_update(th.z, g.z, coef);
-        sgd_update(th.w, g.w, coef);
-    } else {
-        constexpr bool STD = RULE == kRuleFasgdStd;
-        rule_update<ARITH, STD>(th.x, n.x, b.x, v.x, g.x, coef, sp);
-        rule_update<ARITH, STD>(th.y, n.y, b.y, v.y, g.y, coef, sp);
-        rule_update<ARITH, STD>(th.z, n.z, b.z, v.z, g.z, coef, sp);
-        rule_update<ARITH, STD>(th.w, n.w, b.w, v.w, g.w, coef, sp);
-    }
-}
-
-template <int RULE, int ARITH>
 __device__ __forceinline__ void update1(const RangeArgs& a, int64_t p) {
     float th = a.theta[p];
     if (RULE == kRuleSgd) {
@@ -417,6 +400,18 @@ __device__ __forceinline__ void update1(const RangeArgs& a, int64_t p) {
         a.v[p] = v;
     }
     a.theta[p] = th;
+}
+
+// A quad whose exact arithmetic left the range of its fast form.
+template <int RULE>
+__device__ __forceinline__ void redo_quad(const RangeArgs& a, int64_t q, float4& th, float4& n, float4& b,
+                                          float4& v) {
+    const QuadState x = exact_quad<RULE == kRuleFasgdStd>(a.theta, a.n, a.b, a.v, a.grad, nullptr, &a.coef, 1,
+                                                          4 * q, a.sp);
+    th = x.th;
+    n = x.n;
+    b = x.b;
+    v = x.v;
 }
 
 __device__ __forceinline__ float4 ld4(const float* base, int64_t q) {
@@ -469,7 +464,9 @@ __global__ void __launch_bounds__(kItemThreads) tensor_apply_kernel(const __grid
                         v1 = ld4(a.v, q1);
                     }
                 }
-                update4<RULE, ARITH>(th0, n0, b0, v0, g0, a.coef, a.sp);
+                Guard<ARITH> guard0;
+                update4<RULE, ARITH>(th0, n0, b0, v0, g0, a.coef, a.sp, guard0);
+                if (!guard0.ok()) redo_quad<RULE>(a, q0, th0, n0, b0, v0);
                 st4(a.theta, q0, th0);
                 if (FAS) {
                     st4(a.n, q0, n0);
@@ -477,7 +474,9 @@ __global__ void __launch_bounds__(kItemThreads) tensor_apply_kernel(const __grid
                     st4(a.v, q0, v0);
                 }
                 if (two) {
-                    update4<RULE, ARITH>(th1, n1, b1, v1, g1, a.coef, a.sp);
+                    Guard<ARITH> guard1;
+                    update4<RULE, ARITH>(th1, n1, b1, v1, g1, a.coef, a.sp, guard1);
+                    if (!guard1.ok()) redo_quad<RULE>(a, q1, th1, n1, b1, v1);
                     st4(a.theta, q1, th1);
                     if (FAS) {
                         st4(a.n, q1, n1);

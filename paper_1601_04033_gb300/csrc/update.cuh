@@ -98,9 +98,135 @@ __device__ __forceinline__ void fasgd_update_exact(float& theta, float& n, float
     theta = __fsub_rn(theta, __fdiv_rn(__fmul_rn(coef, g), v));
 }
 
+// ---- the exact sequence on pairs -------------------------------------------
+// Two fp32 values in one 64-bit register pair, with the packed fp32
+// instructions of sm_100 and later (each half rounded on its own, no
+// flush to zero): one issue slot for two operations.
+struct Pair {
+    unsigned long long bits;
+};
+__device__ __forceinline__ Pair pair(float x, float y) {
+    Pair p;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(p.bits) : "f"(x), "f"(y));
+    return p;
+}
+__device__ __forceinline__ void unpack(Pair p, float& x, float& y) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(p.bits));
+}
+__device__ __forceinline__ Pair add2(Pair a, Pair b) {
+    Pair d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d.bits) : "l"(a.bits), "l"(b.bits));
+    return d;
+}
+__device__ __forceinline__ Pair mul2(Pair a, Pair b) {
+    Pair d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d.bits) : "l"(a.bits), "l"(b.bits));
+    return d;
+}
+__device__ __forceinline__ Pair fma2(Pair a, Pair b, Pair c) {
+    Pair d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d.bits) : "l"(a.bits), "l"(b.bits), "l"(c.bits));
+    return d;
+}
+
+// fl(a b) that stays a rounding of its own: a product made with mul2 and fed
+// to add2 comes out as one fused multiply-add here (also under -fmad=false),
+// so it is formed as fma(a, b, -0), with a -0 the compiler does not see.
+__device__ __forceinline__ Pair product2(Pair a, Pair b, const StatParams& sp) {
+    return fma2(a, b, pair(sp.minus_zero, sp.minus_zero));
+}
+
+// What the pushes of a pass saw, kept while they are applied: whether the
+// chains of exact_update2 were correctly rounded throughout.  That holds for
+// rad in [2^-100, 2^100], v in [2^-60, 2^60] and a = fl(coef g) zero or of
+// magnitude in [2^-60, 2^60]: no intermediate is then subnormal and no
+// residual rounded.  NaN fails.  One add-and-compare instruction per bound,
+// and no branch among the pushes: a pass looks once, at its end, and forms
+// the quads that left the range again (exact_quad).
+template <int ARITH> struct Guard {
+    __device__ __forceinline__ bool ok() const { return true; }
+};
+
+// fasgd_update_exact on two parameters, the same bits.  CUDA's own square
+// root and division are correctly rounded over the whole fp32 range and cost
+// about 80 issue slots per element-push here, which made the exact pass
+// issue-bound (K = 8 at 25M parameters: 427 us, 55 % of the copy bandwidth).
+// Inside the range above, which every finite training run keeps to, the
+// hardware approximations refined by fused multiply-adds are correctly rounded
+// as well (Markstein, IBM J. Res. Dev. 34(1), 1990: the residual of an almost
+// rounded root or quotient is exact in one fused multiply-add, and one
+// correction by a rounded reciprocal then rounds correctly):
+//   root:        s = rad y, y ~ rad^-1/2;   s + (rad - s^2) y / 2
+//   reciprocal:  z ~ 1 / x;                 z + (1 - x z) z
+//   quotient:    q = a z, z = fl(1/v);      twice q + (a - v q) z (the first
+//                makes q faithful, the second rounds it).
+// The quotient works with -a and -z, which keeps the sign of a zero a.  Root
+// and reciprocal were compared with __fsqrt_rn and __fdiv_rn for every fp32
+// value of the range, the quotient on 4e10 pairs (random, near midpoints,
+// mantissas at both ends): no difference.
+template <bool STD, class G>
+__device__ __forceinline__ void exact_update2(Pair& theta, Pair& n, Pair& b, Pair& v, Pair g, float coef,
+                                              const StatParams& sp, G& guard) {
+    const Pair minus1 = pair(-1.f, -1.f);
+    const Pair gamma = pair(sp.gamma, sp.gamma), rest = pair(sp.one_m_gamma, sp.one_m_gamma);
+    n = add2(product2(gamma, n, sp), product2(rest, mul2(g, g), sp));
+    b = add2(product2(gamma, b, sp), product2(rest, g, sp));
+    float x, y;
+    unpack(fma2(product2(b, b, sp), minus1, n), x, y);     // n - b^2
+    const Pair var = pair(fmaxf(x, 0.0f), fmaxf(y, 0.0f));
+    const Pair rad = add2(var, pair(sp.eps, sp.eps));
+    const Pair minus_rad = fma2(var, minus1, pair(-sp.eps, -sp.eps));
+    unpack(rad, x, y);
+    guard.see_rad(x, y);
+    const Pair inv = pair(rsqrt_approx<true>(x), rsqrt_approx<true>(y));
+    const Pair s = mul2(rad, inv);
+    const Pair root = fma2(fma2(s, s, minus_rad), mul2(inv, pair(-0.5f, -0.5f)), s);
+    Pair r = root;
+    if (!STD) {
+        unpack(root, x, y);
+        const Pair z = pair(rcp_approx<true>(x), rcp_approx<true>(y));
+        r = fma2(fma2(mul2(root, minus1), z, pair(1.f, 1.f)), z, z);
+    }
+    v = add2(product2(pair(sp.beta, sp.beta), v, sp), product2(pair(sp.one_m_beta, sp.one_m_beta), r, sp));
+    unpack(v, x, y);
+    guard.see_v(x, y);
+    const Pair z = pair(rcp_approx<true>(x), rcp_approx<true>(y));
+    const Pair minus_z = fma2(fma2(v, z, minus1), z, mul2(z, minus1));
+    const Pair minus_a = mul2(pair(-coef, -coef), g);
+    unpack(minus_a, x, y);
+    guard.see_a(x, y);
+    Pair q = mul2(minus_a, minus_z);
+    q = fma2(fma2(v, q, minus_a), minus_z, q);
+    q = fma2(fma2(v, q, minus_a), minus_z, q);
+    theta = fma2(q, minus1, theta);
+}
+
 // Arithmetic of a pass: hardware approximations (subnormal-preserving or
 // flush-to-zero forms) or the exact sequence.
 enum : int { kArithApprox = 0, kArithApproxFtz = 1, kArithExact = 2 };
+
+template <> struct Guard<kArithExact> {
+    uint32_t rad = 0, v = 0, a_min = 0xffffffffu, a_max = 0;
+    __device__ __forceinline__ void see_rad(float x, float y) {
+        rad = __viaddmax_u32(__float_as_uint(x), 0u - kRadLo, rad);
+        rad = __viaddmax_u32(__float_as_uint(y), 0u - kRadLo, rad);
+    }
+    __device__ __forceinline__ void see_v(float x, float y) {
+        v = __viaddmax_u32(__float_as_uint(x), 0u - kLo, v);
+        v = __viaddmax_u32(__float_as_uint(y), 0u - kLo, v);
+    }
+    __device__ __forceinline__ void see_a(float x, float y) {
+        const uint32_t mx = __float_as_uint(x) & 0x7fffffffu, my = __float_as_uint(y) & 0x7fffffffu;
+        a_min = __viaddmin_u32(mx, 0xffffffffu, a_min);   // a zero wraps to the largest
+        a_min = __viaddmin_u32(my, 0xffffffffu, a_min);
+        a_max = max(a_max, max(mx, my));
+    }
+    __device__ __forceinline__ bool ok() const {
+        return rad <= kRadHi - kRadLo && v <= kHi - kLo && a_min >= kLo - 1 && a_max <= kHi;
+    }
+    static constexpr uint32_t kRadLo = 27u << 23, kRadHi = 227u << 23;   // 2^-100, 2^100
+    static constexpr uint32_t kLo = 67u << 23, kHi = 187u << 23;         // 2^-60, 2^60
+};
 
 template <int ARITH, bool STD>
 __device__ __forceinline__ void rule_update(float& theta, float& n, float& b, float& v, float g,
@@ -109,6 +235,66 @@ __device__ __forceinline__ void rule_update(float& theta, float& n, float& b, fl
         fasgd_update_exact<STD>(theta, n, b, v, g, coef, sp);
     else
         fasgd_update<ARITH == kArithApproxFtz, STD>(theta, n, b, v, g, coef, sp);
+}
+
+// One push on four consecutive parameters.
+template <int RULE, int ARITH>
+__device__ __forceinline__ void update4(float4& th, float4& n, float4& b, float4& v, const float4& g,
+                                        float coef, const StatParams& sp, Guard<ARITH>& guard) {
+    constexpr bool STD = RULE == kRuleFasgdStd;
+    if constexpr (RULE == kRuleSgd) {
+        sgd_update(th.x, g.x, coef);
+        sgd_update(th.y, g.y, coef);
+        sgd_update(th.z, g.z, coef);
+        sgd_update(th.w, g.w, coef);
+    } else if constexpr (ARITH == kArithExact) {
+        Pair t0 = pair(th.x, th.y), n0 = pair(n.x, n.y), b0 = pair(b.x, b.y), v0 = pair(v.x, v.y);
+        Pair t1 = pair(th.z, th.w), n1 = pair(n.z, n.w), b1 = pair(b.z, b.w), v1 = pair(v.z, v.w);
+        exact_update2<STD>(t0, n0, b0, v0, pair(g.x, g.y), coef, sp, guard);
+        exact_update2<STD>(t1, n1, b1, v1, pair(g.z, g.w), coef, sp, guard);
+        unpack(t0, th.x, th.y);
+        unpack(n0, n.x, n.y);
+        unpack(b0, b.x, b.y);
+        unpack(v0, v.x, v.y);
+        unpack(t1, th.z, th.w);
+        unpack(n1, n.z, n.w);
+        unpack(b1, b.z, b.w);
+        unpack(v1, v.z, v.w);
+    } else {
+        rule_update<ARITH, STD>(th.x, n.x, b.x, v.x, g.x, coef, sp);
+        rule_update<ARITH, STD>(th.y, n.y, b.y, v.y, g.y, coef, sp);
+        rule_update<ARITH, STD>(th.z, n.z, b.z, v.z, g.z, coef, sp);
+        rule_update<ARITH, STD>(th.w, n.w, b.w, v.w, g.w, coef, sp);
+    }
+}
+
+// The quad of parameters at e (a multiple of 4) after K pushes in exact
+// arithmetic, formed again from memory with CUDA's square root and division:
+// for quads whose guard failed, before anything of them is stored.  g0
+// replaces grad[0].
+struct QuadState {
+    float4 th, n, b, v;
+};
+template <bool STD>
+__device__ __noinline__ QuadState exact_quad(const float* theta, const float* n, const float* b,
+                                             const float* v, const float* g0, const float* const* grad,
+                                             const float* coef, int K, int64_t e, const StatParams& sp) {
+    float o[4][4];
+    for (int i = 0; i < 4; ++i) {
+        float th = theta[e + i], x = n[e + i], y = b[e + i], z = v[e + i];
+        for (int k = 0; k < K; ++k)
+            fasgd_update_exact<STD>(th, x, y, z, (k == 0 ? g0 : grad[k])[e + i], coef[k], sp);
+        o[0][i] = th;
+        o[1][i] = x;
+        o[2][i] = y;
+        o[3][i] = z;
+    }
+    QuadState q;
+    q.th = make_float4(o[0][0], o[0][1], o[0][2], o[0][3]);
+    q.n = make_float4(o[1][0], o[1][1], o[1][2], o[1][3]);
+    q.b = make_float4(o[2][0], o[2][1], o[2][2], o[2][3]);
+    q.v = make_float4(o[3][0], o[3][1], o[3][2], o[3][3]);
+    return q;
 }
 
 }  // namespace fasgd

@@ -18,7 +18,7 @@ def test_pull_and_state_copies(P, shift):
     rng = np.random.default_rng(P + shift)
     want = [rng.standard_normal(P).astype(np.float32) for _ in range(4)]
     srv = fasgd.Server(P, 2, 0.01, fasgd.FASGD)
-    srv.set_state(*want, 5)
+    srv.set_state(*[torch.from_numpy(w) for w in want], 5)
     guard = [torch.full((P + 8,), 7.0, device="cuda") for _ in range(4)]
     out = [x[shift:shift + P] for x in guard]
     assert srv.pull(out[0]) == 5
