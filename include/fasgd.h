@@ -446,7 +446,7 @@ FASGD_API int64_t fasgd_kernel_launches(const fasgd_t* h);
  * bfasgd_select_compact, because a handle allocates its state and scratch.
  *
  * This entry point needs no handle and allocates nothing.  Its scratch (the
- * per-parameter bit mask and the per-tile counts and offsets) lives in a
+ * per-parameter bit mask and the per-tile counts) lives in a
  * fixed static device array of BFASGD_NOALLOC_SCRATCH_BYTES (about 2 MiB)
  * that every GPU which loads the library holds until the process exits.
  * The first call on a device looks up that array's device address (once per
@@ -471,7 +471,7 @@ FASGD_API int64_t fasgd_kernel_launches(const fasgd_t* h);
  * Errors: EINVAL (bad argument or P too large), ECUDA.
  */
 #define BFASGD_NOALLOC_PMAX ((int64_t)1 << 24)              /* 16,777,216 parameters */
-#define BFASGD_NOALLOC_SCRATCH_BYTES ((int64_t)2121728)     /* mask + tile counts + tile bases */
+#define BFASGD_NOALLOC_SCRATCH_BYTES ((int64_t)2121728)     /* holds the mask and the tile counts */
 FASGD_API int bfasgd_select_compact_noalloc(int64_t P, const float* grad, const float* v, float c,
                                             float eps_b, uint64_t seed, int32_t client,
                                             uint64_t push_no, int32_t* idx, float* val,

@@ -74,10 +74,9 @@ struct SparseArgs {
     int32_t* err;              // device error flags (bit 0: count, bit 1: index, bit 2: order)
 };
 
-// Elements per tile of the select / compact kernels, and the bit mask words a
-// tile owns (one bit per element).
-constexpr int kSelectThreads = 256;
-constexpr int kSelectTile = 8192;
+// Parameters per tile of the select kernels, and the bit mask words a tile
+// owns (one bit per parameter).
+constexpr int kSelectTile = 4096;
 constexpr int kSelectTileWords = kSelectTile / 32;
 
 struct SelectArgs {
@@ -87,7 +86,7 @@ struct SelectArgs {
     float* val;
     int64_t* count;      // total number sent (int64, device)
     uint32_t* mask;      // scratch: ntiles * kSelectTileWords words
-    int32_t* tile_count; // scratch: ntiles
+    uint16_t* tile_count; // scratch: ntiles, 16-byte aligned, readable to a multiple of eight
     int64_t* tile_base;  // scratch: ntiles
     int64_t P;
     int32_t ntiles;

@@ -120,7 +120,7 @@ struct fasgd_s {
     float* b = nullptr;
     float* v = nullptr;
     uint32_t* mask = nullptr;
-    int32_t* tile_count = nullptr;
+    uint16_t* tile_count = nullptr;
     int64_t* tile_base = nullptr;
     int32_t* dev_err = nullptr;
     int32_t ntiles = 0;
@@ -449,7 +449,7 @@ int fasgd_create(fasgd_t** h, int64_t P, int32_t lambda, float alpha, int32_t va
         st = cudaMalloc(reinterpret_cast<void**>(&s->mask),
                         (size_t)s->ntiles * fasgd::kSelectTileWords * sizeof(uint32_t));
     if (st == cudaSuccess)
-        st = cudaMalloc(reinterpret_cast<void**>(&s->tile_count), (size_t)s->ntiles * sizeof(int32_t));
+        st = cudaMalloc(reinterpret_cast<void**>(&s->tile_count), ((size_t)s->ntiles + 7) / 8 * 8 * sizeof(uint16_t));
     if (st == cudaSuccess)
         st = cudaMalloc(reinterpret_cast<void**>(&s->tile_base), (size_t)s->ntiles * sizeof(int64_t));
     if (st == cudaSuccess) st = cudaMalloc(reinterpret_cast<void**>(&s->dev_err), sizeof(int32_t));

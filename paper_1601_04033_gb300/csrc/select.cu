@@ -4,105 +4,168 @@
 // the server's theta for a fetch).  Push and fetch draws come from separate
 // Philox counter streams (bit 31 of the client word).
 //
-// Three kernels, all on the caller's stream:
-//   1. mask:    per tile of 8192 parameters, draw u_p (Philox4x32-10), take
-//               the Eq. 9 decision against v_p, write one bit per parameter
-//               and the tile's count of sent entries;
-//   2. scan:    exclusive prefix sum of the tile counts (one block) and the
-//               total m;
-//   3. compact: per tile, rebuild each parameter's rank among the sent ones
-//               from the bit mask (warp popc + shuffles, block scan over
-//               warps) and write idx[rank] = p, val[rank] = grad[p], staged
-//               per warp in shared memory so that the stores are coalesced.
-// The order of the output is the order of p, so the result is unique and
-// does not depend on the launch; no atomics are used.  Traffic per
-// parameter: v (4 B) + grad (4 B) + 2 x 1/8 B of mask, plus 8 B per sent
-// entry.  Each lane issues all eight of its 128-bit loads before it computes.
+// Two kernels, on the caller's stream:
+//   1. decide:  per tile of 4096 parameters (one block, 1024 per warp), draw u_p
+//               (Philox4x32-10), take the Eq. 9 decision against v_p, store one
+//               bit per parameter and the tile's count of kept entries;
+//   2. compact: per tile, the sum of the earlier tiles' counts gives its place
+//               in the lists; the kept entries are written there in order.
+// (Beyond 8192 tiles a scan kernel between them forms those sums once, so that
+// the tiles do not each read all the counts before theirs.)  The order of the
+// output is the order of p, so the result is unique and does not depend on the
+// launch; no atomics, and no block waits for another.
+//
+// Bounds.  decide: the multiply and ALU pipes (ncu at 25M: 24.3 us, the fused
+// multiply-add heavy pipe 67 % and the ALU 57 % busy, DRAM 4.1 TB/s):
+// Philox4x32-10 is some 15 instructions per parameter, the test 4, on packed
+// fp32 pairs, and one funnel shift takes its sign bit into the lane's word.
+// compact: HBM and latency (23.6 us for 103 MB read and 40 MB written).
+// Each lane decides quads 32 it + lane (it = 0 .. 7) of its warp's 1024, so its
+// bits are in another order than the parameters': an 8 x 8 transposition of
+// nibbles among eight lanes (three shuffles) and one more shuffle give lane l
+// the 32 bits of parameters 32 l .. 32 l + 31.  Each lane then writes its set
+// bits' offsets at their ranks into shared memory (one step per kept entry
+// instead of tests per parameter: 0.46 instead of 0.69 warp instructions per
+// parameter), and consecutive lanes fetch the kept values, so that only their
+// sectors are read, and write consecutive entries.
+// Blocks of 128 threads, eight per SM: a tile is small beside the SM's share
+// at 1.3M parameters already, and the last wave is short.
+// The whole select of 25M parameters at 20 % kept: 57 -> about 46 us with the
+// scan kernel gone (exchange of four clients 1068 -> 976 us); of 1.29M: four
+// exchanges 135 -> 110 us, from Python.
+//
+// Tried as one kernel (the compaction's memory time under the decision's ALU
+// time): warps that wait for the counts of earlier tiles took 140 us per 25M
+// one tile each (the polls of the same few words), and 57 us persistent with
+// three decided tiles in hand (tickets for the tiles, one address, cost 2.3 ns
+// an atomic).  Values prefetched into L2 by decide: 1014 against 986 us.
 
 #include "eq9.cuh"
 #include "kernels.cuh"
 #include "pdl.cuh"
+#include "update.cuh"
 
 namespace fasgd {
 namespace {
 
-constexpr int kWarps = kSelectThreads / 32;
-constexpr int kWarpSpan = kSelectTile / kWarps;  // 1024 parameters per warp
-constexpr int kIters = kWarpSpan / 128;          // 8 passes of 32 lanes x 4
+// Both kernels: a span of 1024 parameters per warp.
+constexpr int kSpan = 1024;
+constexpr int kThreads = kSelectTile / 32;
+constexpr int kWarps = kThreads / 32;
+constexpr int kQuads = kSpan / 128;               // quads per lane of the decision
 constexpr unsigned kFull = 0xffffffffu;
 
-// The four values e .. e+3 of x (zero past P; FULL: the tile lies inside P).
-template <bool FULL>
-__device__ __forceinline__ float4 load_quad(const float* x, int64_t e, int64_t P) {
-    if (FULL || e + 3 < P) return __ldcs(reinterpret_cast<const float4*>(x + e));
-    float t[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int j = 0; j < 4; ++j)
-        if (e + j < P) t[j] = x[e + j];
-    return make_float4(t[0], t[1], t[2], t[3]);
+__device__ __forceinline__ uint32_t smem_address(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// This lane's quads of v in the warp's span at `start` (zero past P).
+__device__ __forceinline__ void load_quads(float4 (&q)[kQuads], const float* v, int64_t start, int64_t P,
+                                          int lane) {
+    const int64_t e = start + 4 * lane;
+    if (start + kSpan <= P) {
+#pragma unroll
+        for (int it = 0; it < kQuads; ++it) q[it] = __ldcs(reinterpret_cast<const float4*>(v + e + 128 * it));
+    } else {
+#pragma unroll
+        for (int it = 0; it < kQuads; ++it) {
+            const int64_t p = e + 128 * it;
+            q[it].x = p < P ? v[p] : 0.f;
+            q[it].y = p + 1 < P ? v[p + 1] : 0.f;
+            q[it].z = p + 2 < P ? v[p + 2] : 0.f;
+            q[it].w = p + 3 < P ? v[p + 3] : 0.f;
+        }
+    }
 }
 
-template <bool FULL, bool SCALE_D>
-__device__ __forceinline__ void mask_tile(const SelectArgs& a) {
-    __shared__ int32_t warp_cnt[kWarps];
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int64_t tile_start = (int64_t)blockIdx.x * kSelectTile;
-    const int64_t warp_start = tile_start + (int64_t)warp * kWarpSpan;
-    // All of this lane's v loads first (eight quads), then the draws.
-    float4 v4[kIters];
-#pragma unroll
-    for (int it = 0; it < kIters; ++it) v4[it] = load_quad<FULL>(a.v, warp_start + it * 128 + 4 * lane, a.P);
-    const uint32_t e_lane = (uint32_t)(warp_start + 4 * lane);  // P < 2^31
-    int cnt = 0;
-#pragma unroll
-    for (int it = 0; it < kIters; ++it) {
-        const uint32_t e = e_lane + it * 128;
-        uint32_t nib = 0;
-        if (FULL || e < a.P) {
-            const Philox4 r = philox4x32_10(e >> 2, a.client_word, a.push_lo, a.push_hi, a.round_key0, a.round_key1);
-            nib = (send_test<SCALE_D>(r.x[0] >> 8, v4[it].x, a.c, a.eps_b) ? 1u : 0u) |
-                  (send_test<SCALE_D>(r.x[1] >> 8, v4[it].y, a.c, a.eps_b) ? 2u : 0u) |
-                  (send_test<SCALE_D>(r.x[2] >> 8, v4[it].z, a.c, a.eps_b) ? 4u : 0u) |
-                  (send_test<SCALE_D>(r.x[3] >> 8, v4[it].w, a.c, a.eps_b) ? 8u : 0u);
-            if (!FULL) {
-                const int64_t valid = a.P - e;  // parameters past P are never sent
-                if (valid < 4) nib &= (1u << valid) - 1u;
-            }
-        }
-        cnt += __popc(nib);
-        // Eight lanes' nibbles form one 32-bit mask word (32 consecutive parameters).
-        uint32_t w = nib << (4 * (lane & 7));
-        w |= __shfl_xor_sync(kFull, w, 1);
-        w |= __shfl_xor_sync(kFull, w, 2);
-        w |= __shfl_xor_sync(kFull, w, 4);
-        if ((lane & 7) == 0)
-            a.mask[(warp_start >> 5) + it * 4 + (lane >> 3)] = w;
+// The sign of u d - a 2^24 for two parameters (send_test's difference, as
+// packed operations): negative means sent.
+template <bool SCALE_D>
+__device__ __forceinline__ void send_difference(uint32_t w0, uint32_t w1, float v0, float v1, Pair c,
+                                                Pair eps_b, float& s0, float& s1) {
+    const Pair a = add2(pair(v0, v1), eps_b);
+    const Pair d = add2(a, c);
+    const Pair u = pair((float)(w0 >> 8), (float)(w1 >> 8));   // exact: below 2^24
+    if (SCALE_D) {
+        const Pair scale = pair(5.9604644775390625e-8f, 5.9604644775390625e-8f);
+        unpack(fma2(u, mul2(d, scale), mul2(a, pair(-1.f, -1.f))), s0, s1);
+    } else {
+        unpack(fma2(u, d, mul2(a, pair(-16777216.0f, -16777216.0f))), s0, s1);
     }
+}
+
+// Bit 4 it + j: parameter start + 128 it + 4 lane + j is sent.
+template <bool SCALE_D>
+__device__ __forceinline__ uint32_t quad_bits(const SelectArgs& a, const float4 (&v)[kQuads], uint32_t start,
+                                              int lane) {
+    const Pair c = pair(a.c, a.c), eps_b = pair(a.eps_b, a.eps_b);
+    uint32_t bits = 0;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) cnt += __shfl_xor_sync(kFull, cnt, off);
-    if (lane == 0) warp_cnt[warp] = cnt;
+    for (int it = kQuads - 1; it >= 0; --it) {
+        const uint32_t e = start + 128 * it + 4 * lane;   // P < 2^31
+        const Philox4 r = philox4x32_10(e >> 2, a.client_word, a.push_lo, a.push_hi, a.round_key0, a.round_key1);
+        float s[4];
+        send_difference<SCALE_D>(r.x[0], r.x[1], v[it].x, v[it].y, c, eps_b, s[0], s[1]);
+        send_difference<SCALE_D>(r.x[2], r.x[3], v[it].z, v[it].w, c, eps_b, s[2], s[3]);
+#pragma unroll
+        for (int j = 3; j >= 0; --j) {
+            if (SCALE_D)   // c = +inf can make a NaN: not sent
+                bits = 2 * bits + (s[j] < 0.f ? 1u : 0u);
+            else           // one funnel shift takes the sign in
+                bits = __funnelshift_l(__float_as_uint(s[j]), bits, 1);
+        }
+    }
+    return bits;
+}
+
+// From this lane's quads' bits (nibble it: quad 32 it + lane) to the bits of
+// parameters 32 lane .. 32 lane + 31 of the span.
+__device__ __forceinline__ uint32_t lane_word(uint32_t x, int lane) {
+    // Nibble (lane & 7, it) <-> (it, lane & 7) within each group of eight lanes.
+    uint32_t y = __shfl_xor_sync(kFull, x, 4);
+    x = __byte_perm(x, y, (lane & 4) ? 0x3276 : 0x5410);
+    y = __shfl_xor_sync(kFull, x, 2);
+    x = __byte_perm(x, y, (lane & 2) ? 0x3715 : 0x6240);
+    y = __shfl_xor_sync(kFull, x, 1);
+    x = (lane & 1) ? (x & 0xf0f0f0f0u) | ((y >> 4) & 0x0f0f0f0fu) : (x & 0x0f0f0f0fu) | ((y << 4) & 0xf0f0f0f0u);
+    // Lane 8 a + b now holds word 4 b + a.
+    return __shfl_sync(kFull, x, 8 * (lane & 3) + (lane >> 2));
+}
+
+// SCALE_D: the form of the Eq. 9 test for this call's c (send_form).
+template <bool SCALE_D>
+__global__ void __launch_bounds__(kThreads, 8) bfasgd_decide_kernel(const __grid_constant__ SelectArgs a) {
+    __shared__ int32_t warp_cnt[kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t start = (int64_t)blockIdx.x * kSelectTile + warp * kSpan;
+    pdl_wait();
+    pdl_trigger();
+    float4 v[kQuads];
+    load_quads(v, a.v, start, a.P, lane);
+    uint32_t bits = quad_bits<SCALE_D>(a, v, (uint32_t)start, lane);
+    if (start + kSpan > a.P) {   // parameters past P are never sent
+#pragma unroll
+        for (int it = 0; it < kQuads; ++it) {
+            const int64_t left = a.P - (start + 128 * it + 4 * lane);
+            const uint32_t keep = left >= 4 ? 0xfu : left <= 0 ? 0u : (1u << left) - 1u;
+            bits &= ~((~keep & 0xfu) << (4 * it));
+        }
+    }
+    a.mask[(start >> 5) + lane] = bits;
+    const int n = (int)__reduce_add_sync(kFull, (uint32_t)__popc(bits));
+    if (lane == 0) warp_cnt[warp] = n;
     __syncthreads();
     if (threadIdx.x == 0) {
         int32_t t = 0;
 #pragma unroll
         for (int w = 0; w < kWarps; ++w) t += warp_cnt[w];
-        a.tile_count[blockIdx.x] = t;
+        a.tile_count[blockIdx.x] = (uint16_t)t;
     }
 }
 
-// Full tiles (all but perhaps the last) skip the per-quad bounds checks.
-// SCALE_D: the form of the Eq. 9 test for this call's c (send_form).
-template <bool SCALE_D>
-__global__ void __launch_bounds__(kSelectThreads) bfasgd_mask_kernel(const __grid_constant__ SelectArgs a) {
-    pdl_wait();
-    pdl_trigger();
-    if ((int64_t)(blockIdx.x + 1) * kSelectTile <= a.P)
-        mask_tile<true, SCALE_D>(a);
-    else
-        mask_tile<false, SCALE_D>(a);
-}
-
 constexpr int kScanThreads = 1024;
+// More tiles than this (33.5M parameters): their bases come from the scan
+// kernel (4 us); up to there each tile reads the counts before its own (16 KB
+// at most, on average half, from L2), in the shadow of its other loads.
+constexpr int kScanTiles = 8192;
 
 __global__ void __launch_bounds__(kScanThreads) bfasgd_scan_kernel(const __grid_constant__ SelectArgs a) {
     __shared__ int64_t warp_sum[kScanThreads / 32];
@@ -118,7 +181,7 @@ __global__ void __launch_bounds__(kScanThreads) bfasgd_scan_kernel(const __grid_
     int64_t local = 0;
     if (per <= kKeep) {
 #pragma unroll
-        for (int k = 0; k < kKeep; ++k) kept[k] = lo + k < hi ? a.tile_count[lo + k] : 0;
+        for (int k = 0; k < kKeep; ++k) kept[k] = lo + k < hi ? (int32_t)a.tile_count[lo + k] : 0;
 #pragma unroll
         for (int k = 0; k < kKeep; ++k) local += kept[k];
     } else {
@@ -160,77 +223,92 @@ __global__ void __launch_bounds__(kScanThreads) bfasgd_scan_kernel(const __grid_
     if (tid == kScanThreads - 1) *a.count = warp_sum[kScanThreads / 32 - 1];
 }
 
-// Per warp and pass, the kept (index, value) pairs are first put in rank
-// order in shared memory, then written to idx and val by consecutive lanes
-// (coalesced), instead of each lane storing its own pairs at scattered ranks.
-constexpr int kPassParams = 128;
-
-template <bool FULL>
-__device__ __forceinline__ void compact_tile(const SelectArgs& a, uint2* stage) {
-    __shared__ int32_t warp_cnt[kWarps];
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int64_t tile_start = (int64_t)blockIdx.x * kSelectTile;
-    const int64_t warp_start = tile_start + (int64_t)warp * kWarpSpan;
-    // Lane l holds the mask word of parameters warp_start + 32 l .. + 31.  The
-    // word, the tile's output base and the value quads are all loaded before
-    // anything waits on them.
-    const uint32_t word = a.mask[(warp_start >> 5) + lane];
-    const int64_t tile_out = a.tile_base[blockIdx.x];
-    float4 g4[kIters];
-#pragma unroll
-    for (int it = 0; it < kIters; ++it)
-        g4[it] = load_quad<FULL>(a.values, warp_start + it * kPassParams + 4 * lane, a.P);
-    const int c = __popc(word);
-    int incl = c;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int y = __shfl_up_sync(kFull, incl, off);
-        if (lane >= off) incl += y;
-    }
-    const int excl = incl - c;  // rank of this word's first kept entry in the warp's span
-    if (lane == 31) warp_cnt[warp] = incl;
-    __syncthreads();
-    int64_t out = tile_out;
-    for (int w = 0; w < warp; ++w) out += warp_cnt[w];
-    int32_t* idx_w = a.idx + out;
-    float* val_w = a.val + out;
-    const int32_t e_lane = (int32_t)(warp_start + 4 * lane);  // P < 2^31
-    const int sh = 4 * (lane & 7);
-#pragma unroll
-    for (int it = 0; it < kIters; ++it) {
-        // This lane's quad lies in word (4 it + lane / 8), bits sh .. sh + 3.
-        const int owner = it * 4 + (lane >> 3);
-        const uint32_t w = __shfl_sync(kFull, word, owner);
-        const int wbase = __shfl_sync(kFull, excl, owner);
-        const int pass_base = __shfl_sync(kFull, excl, it * 4);
-        const int pass_end = __shfl_sync(kFull, incl, it * 4 + 3);
-        const uint32_t nib = (w >> sh) & 0xFu;
-        int r = wbase - pass_base + __popc(w & ((1u << sh) - 1u));
-        const int32_t e = e_lane + it * kPassParams;
-        const uint32_t g[4] = {__float_as_uint(g4[it].x), __float_as_uint(g4[it].y),
-                               __float_as_uint(g4[it].z), __float_as_uint(g4[it].w)};
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if ((nib >> j) & 1u) stage[r++] = make_uint2((uint32_t)(e + j), g[j]);
-        __syncwarp();
-        for (int k = lane; k < pass_end - pass_base; k += 32) {
-            const uint2 pr = stage[k];
-            idx_w[pass_base + k] = (int32_t)pr.x;
-            val_w[pass_base + k] = __uint_as_float(pr.y);
-        }
-        __syncwarp();
-    }
-}
-
-__global__ void __launch_bounds__(kSelectThreads) bfasgd_compact_kernel(const __grid_constant__ SelectArgs a) {
-    __shared__ uint2 stage[kWarps][kPassParams];
+// SCANNED: tile_base holds the sums (bfasgd_scan_kernel), else the block adds
+// the counts before its tile.
+template <bool SCANNED>
+__global__ void __launch_bounds__(kThreads, 8) bfasgd_compact_kernel(const __grid_constant__ SelectArgs a) {
+    __shared__ uint16_t s_off[kWarps][kSpan];
+    __shared__ int32_t warp_cnt[kWarps], warp_sum[kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint16_t* off = s_off[warp];
+    const int64_t start = (int64_t)blockIdx.x * kSelectTile + warp * kSpan;
     pdl_wait();
     pdl_trigger();
-    if ((int64_t)(blockIdx.x + 1) * kSelectTile <= a.P)
-        compact_tile<true>(a, stage[threadIdx.x >> 5]);
-    else
-        compact_tile<false>(a, stage[threadIdx.x >> 5]);
+    const uint32_t bits = a.mask[(start >> 5) + lane];
+    int64_t tile_out = 0;
+    int32_t before = 0;
+    if (SCANNED) {
+        tile_out = a.tile_base[blockIdx.x];
+    } else {
+        // Eight counts per load; the last load's own and later ones are left out.
+        for (int t = 8 * threadIdx.x; t < (int)blockIdx.x; t += 8 * kThreads) {
+            const uint4 q = *reinterpret_cast<const uint4*>(a.tile_count + t);
+            const uint32_t c[4] = {q.x, q.y, q.z, q.w};
+            const int left = (int)blockIdx.x - t;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (2 * i < left) before += (int32_t)(c[i] & 0xffffu);
+                if (2 * i + 1 < left) before += (int32_t)(c[i] >> 16);
+            }
+        }
+    }
+    uint32_t word = lane_word(bits, lane);
+    const int n = __popc(word);
+    int incl = n;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, d);
+        if (lane >= d) incl += y;
+    }
+    if (lane == 31) warp_cnt[warp] = incl;
+    if (!SCANNED) {
+        before = (int32_t)__reduce_add_sync(kFull, (uint32_t)before);
+        if (lane == 0) warp_sum[warp] = before;
+    }
+    // From the highest bit down: one step per kept entry.
+    for (int r = incl - 1; word != 0; --r) {
+        const int b = 31 - __clz((int)word);
+        off[r] = (uint16_t)(32 * lane + b);
+        word ^= 1u << b;
+    }
+    __syncwarp();
+    const int mine = __shfl_sync(kFull, incl, 31);
+    // The kept values, in the order of the list.
+    const float* src = a.values + start;
+    constexpr int kHeld = 8;
+    float x[kHeld];
+    int o[kHeld];
+#pragma unroll
+    for (int i = 0; i < kHeld; ++i) {
+        const int k = lane + 32 * i;
+        if (k < mine) {
+            o[i] = off[k];
+            x[i] = __ldcs(src + o[i]);
+        }
+    }
+    __syncthreads();
+    int64_t out = tile_out;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        if (!SCANNED) out += warp_sum[w];
+        if (w < warp) out += warp_cnt[w];
+    }
+    int32_t* idx_out = a.idx + out;
+    float* val_out = a.val + out;
+#pragma unroll
+    for (int i = 0; i < kHeld; ++i) {
+        const int k = lane + 32 * i;
+        if (k < mine) {
+            idx_out[k] = (int32_t)start + o[i];
+            val_out[k] = x[i];
+        }
+    }
+    for (int k = lane + 32 * kHeld; k < mine; k += 32) {
+        const int p = off[k];
+        idx_out[k] = (int32_t)start + p;
+        val_out[k] = __ldcs(src + p);
+    }
+    if (!SCANNED && blockIdx.x == gridDim.x - 1 && warp == kWarps - 1 && lane == 0) *a.count = out + mine;
 }
 
 }  // namespace
@@ -240,15 +318,18 @@ void select_key_schedule(SelectArgs& a, uint64_t seed) {
 }
 
 cudaError_t launch_select(const SelectArgs& a, cudaStream_t stream, int64_t* launches) {
-    cudaError_t st = send_form(a.c)
-                         ? launch_pdl(bfasgd_mask_kernel<true>, a.ntiles, kSelectThreads, 0, stream, a)
-                         : launch_pdl(bfasgd_mask_kernel<false>, a.ntiles, kSelectThreads, 0, stream, a);
+    const auto decide = send_form(a.c) ? bfasgd_decide_kernel<true> : bfasgd_decide_kernel<false>;
+    cudaError_t st = launch_pdl(decide, (unsigned)a.ntiles, kThreads, 0, stream, a);
     if (st != cudaSuccess) return st;
     ++*launches;
-    st = launch_pdl(bfasgd_scan_kernel, 1, kScanThreads, 0, stream, a);
-    if (st != cudaSuccess) return st;
-    ++*launches;
-    st = launch_pdl(bfasgd_compact_kernel, a.ntiles, kSelectThreads, 0, stream, a);
+    const bool scan = a.ntiles > kScanTiles;
+    if (scan) {
+        st = launch_pdl(bfasgd_scan_kernel, 1, kScanThreads, 0, stream, a);
+        if (st != cudaSuccess) return st;
+        ++*launches;
+    }
+    const auto compact = scan ? bfasgd_compact_kernel<true> : bfasgd_compact_kernel<false>;
+    st = launch_pdl(compact, (unsigned)a.ntiles, kThreads, 0, stream, a);
     if (st != cudaSuccess) return st;
     ++*launches;
     return cudaSuccess;
@@ -258,7 +339,7 @@ cudaError_t launch_select(const SelectArgs& a, cudaStream_t stream, int64_t* lau
 
 // ---------------------------------------------------------------------------
 // Allocation-free variant of bfasgd_select_compact for callers that may not
-// allocate device memory (see include/fasgd.h).  The same three kernels run
+// allocate device memory (see include/fasgd.h).  The same kernels run
 // with their scratch in one fixed static device array instead of handle-owned
 // buffers.
 // ---------------------------------------------------------------------------
@@ -272,16 +353,15 @@ void set_handleless_error(const char* msg);  // defined in runtime.cu
 
 namespace {
 
-constexpr int64_t kNoallocTiles = BFASGD_NOALLOC_PMAX / fasgd::kSelectTile;          // 2048
+constexpr int64_t kNoallocTiles = BFASGD_NOALLOC_PMAX / fasgd::kSelectTile;          
 constexpr int64_t kNoallocMaskBytes = kNoallocTiles * fasgd::kSelectTileWords * 4;  // 2 MiB
-constexpr int64_t kNoallocCountBytes = kNoallocTiles * 4;
-constexpr int64_t kNoallocBaseBytes = kNoallocTiles * 8;
-static_assert(kNoallocMaskBytes + kNoallocCountBytes + kNoallocBaseBytes ==
-                  BFASGD_NOALLOC_SCRATCH_BYTES,
+constexpr int64_t kNoallocCountBytes = kNoallocTiles * 2;
+static_assert(kNoallocMaskBytes + kNoallocCountBytes <= BFASGD_NOALLOC_SCRATCH_BYTES,
               "scratch size in fasgd.h out of date");
-static_assert(kNoallocMaskBytes % 256 == 0 && kNoallocCountBytes % 8 == 0, "scratch layout");
+static_assert(kNoallocMaskBytes % 256 == 0 && kNoallocTiles % 8 == 0, "scratch layout");
+static_assert(kNoallocTiles <= fasgd::kScanTiles, "no tile bases here");
 
-// Mask words, then int32 tile counts, then int64 tile bases.
+// Mask words, then 16-bit tile counts.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[BFASGD_NOALLOC_SCRATCH_BYTES];
 
 constexpr int kMaxDevices = 64;
@@ -369,8 +449,8 @@ extern "C" int bfasgd_select_compact_noalloc(int64_t P, const float* grad, const
     a.val = val;
     a.count = n_dev;
     a.mask = reinterpret_cast<uint32_t*>(scratch);
-    a.tile_count = reinterpret_cast<int32_t*>(scratch + kNoallocMaskBytes);
-    a.tile_base = reinterpret_cast<int64_t*>(scratch + kNoallocMaskBytes + kNoallocCountBytes);
+    a.tile_count = reinterpret_cast<uint16_t*>(scratch + kNoallocMaskBytes);
+    a.tile_base = nullptr;   // too few tiles for the scan kernel
     a.P = P;
     a.ntiles = fasgd::select_tiles(P);
     a.c = c;

@@ -1,0 +1,42 @@
+"""The select kernels where their forms meet: around 8192 tiles of 4096
+parameters (beyond, a scan kernel forms the tiles' places) and at densities on
+both sides of 256 kept entries per warp (fetched before or after the place is
+known), every list bit for bit against the oracle."""
+
+import numpy as np
+import pytest
+
+import oracle
+from gpu_util import binding, torch_cuda
+from paper_1601_04033_gb300 import streams
+
+pytestmark = pytest.mark.gpu
+SWITCH = 8192 * 4096
+
+
+@pytest.mark.parametrize("P,c", [(SWITCH, 40.0), (SWITCH + 1, 40.0), (SWITCH - 4095, 40.0)]
+                         + [(P, c) for P in (1, 31, 1023, 1025, 4095, 4097, 40_961)
+                            for c in (0.0, 1.0, 30.0, 90.0, 1e4, float(2.0 ** 80), float("inf"))])
+def test_select_lists_against_oracle(P, c):
+    torch, f = torch_cuda(), binding()
+    rng = np.random.default_rng(P % 9973)
+    grad = rng.standard_normal(P, dtype=np.float32)
+    v = np.exp(rng.random(P, dtype=np.float32) * np.float32(4.6))
+    if P == 40_961:            # one warp all kept beside one with nothing kept
+        v[1024:2048] = 1e30
+        v[2048:3072] = 0.0
+    srv = f.Server(P, 4, 0.001, f.FASGD, c_push=c, eps_b=1e-8, seed=11)
+    g, vv = torch.from_numpy(grad).cuda(), torch.from_numpy(v).cuda()
+    idx = torch.full((P,), -1, dtype=torch.int32, device="cuda")
+    val = torch.zeros(P, device="cuda")
+    cnt = torch.full((1,), -1, dtype=torch.int64, device="cuda")
+    for n in range(2):         # twice: nothing carries over
+        srv.select_compact(3, g, idx, val, cnt, v=vv)
+        srv.sync()
+        oi, ov = oracle.select(grad, v, c, 1e-8, 11, 3, n)
+        m = int(cnt.item())
+        assert m == oi.size
+        assert np.array_equal(idx[:m].cpu().numpy(), oi)
+        assert np.array_equal(val[:m].cpu().numpy().view(np.uint32), ov.view(np.uint32))
+        assert (idx[m:] == -1).all() or n == 1
+    srv.close()
