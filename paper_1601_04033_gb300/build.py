@@ -13,6 +13,7 @@ import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -53,8 +54,9 @@ def up_to_date() -> bool:
 
 
 def build(force: bool = False, verbose: bool = False, extra_flags: list | None = None) -> str:
-    """Build libfasgd.so if needed; returns its path."""
+    """Build libfasgd.so (and the binding's module) if needed; returns its path."""
     if not force and up_to_date():
+        build_binding()
         return LIB
     os.makedirs(BUILD, exist_ok=True)
     exe = nvcc()
@@ -81,7 +83,33 @@ def build(force: bool = False, verbose: bool = False, extra_flags: list | None =
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, LIB)
+    build_binding(force)
     return LIB
+
+
+BINDING_SRC = os.path.join(PKG, "binding.c")
+BINDING = os.path.join(PKG, "_binding.so")
+
+
+def build_binding(force: bool = False) -> str | None:
+    """Build the CPython module of the binding's hot calls (binding.c) against
+    libfasgd.so; returns its path, or None where Python's headers are not
+    installed (the binding then makes every call through ctypes)."""
+    include = sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(include, "Python.h")):
+        return None
+    newest = max(os.path.getmtime(p) for p in (BINDING_SRC, os.path.join(INCLUDE, "fasgd.h")))
+    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= newest:
+        return BINDING
+    tmp = BINDING + f".tmp{os.getpid()}"
+    cmd = ["gcc", "-O2", "-std=c11", "-Wall", "-Wextra", "-shared", "-fPIC", "-fvisibility=hidden",
+           BINDING_SRC, f"-I{include}", f"-I{INCLUDE}", f"-L{PKG}", "-lfasgd", "-Wl,-rpath,$ORIGIN",
+           "-o", tmp]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"binding build failed:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, BINDING)
+    return BINDING
 
 
 DRIVER_SRC = os.path.join(PKG, "abi_latency.c")

@@ -255,6 +255,18 @@ def fasgd_last_error(h) -> str:
     return s.decode() if s else ""
 
 
+# The hot entry points again, without ctypes' cost per call (binding.c): the
+# same names, arguments and results.  Absent where Python's headers were not
+# installed when the library was built; the functions above then serve.
+try:
+    from . import _binding
+except ImportError:
+    _binding = None
+if _binding is not None:
+    for _name in _binding.install(globals()):
+        globals()[_name] = getattr(_binding, _name)
+
+
 # ---------------------------------------------------------------------------
 # Tensor-level wrapper
 # ---------------------------------------------------------------------------
@@ -264,6 +276,16 @@ def _ptr(t) -> int | None:
     if not t.is_contiguous():
         raise ValueError("tensor must be contiguous")
     return t.data_ptr()
+
+
+def _current_stream() -> int:
+    """torch's current stream on the current device, as an address (without the
+    3 us of building a torch.cuda.Stream object, where torch offers that)."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch._C._cuda_getDevice())
 
 
 def aligned_vectors(data, device="cuda"):
@@ -282,12 +304,11 @@ def aligned_vectors(data, device="cuda"):
 
 def fetch_apply(theta_client, idx, val, n_dev=None, n_max=None, err_dev=None, stream=None):
     """Client side of a B-FASGD fetch (bfasgd_fetch_apply) on torch tensors."""
-    import torch
     if n_max is None:
         n_max = idx.numel()
-    s = stream if stream is not None else torch.cuda.current_stream()
+    s = stream.cuda_stream if stream is not None else _current_stream()
     rc = bfasgd_fetch_apply(theta_client.numel(), _ptr(theta_client), _ptr(idx), _ptr(val),
-                            _ptr(n_dev), n_max, s.cuda_stream, _ptr(err_dev))
+                            _ptr(n_dev), n_max, s, _ptr(err_dev))
     if rc != OK:
         raise FasgdError(rc, fasgd_last_error(None))
 
