@@ -7,29 +7,27 @@
 // for FASGD, the minimum for K pushes (paper Sec. 2.1 protocol, Eq. 1-2 and
 // Eq. 4-8 applied K times).
 //
-// Structure: a persistent kernel, one block per SM, one producer warp and
-// 16 consumer warps.  The parameter range is cut into tiles of 2048; the
-// producer's elected lane stages each tile's state slices and up to 8
-// gradient slices into a shared-memory ring with 1-D bulk async copies
+// Structure: a persistent kernel, one block per SM (or two smaller ones), one
+// producer warp and 16 consumer warps.  The parameter range is cut into tiles
+// of 2048; the producer's elected lane stages each tile's state slices and up
+// to CH gradient slices into a shared-memory ring with 1-D bulk async copies
 // (cp.async.bulk, completion counted on an mbarrier), while the consumer
 // warps compute on the previous stage: each thread takes four consecutive
 // parameters (128-bit shared loads), frees the stage as soon as its inputs
 // are in registers, applies the pushes, and stores the state with 128-bit
-// global stores.  A stage holds up to 8 gradient slices; larger K runs as
-// several stages per tile (the state travels with the first one only).  The
-// last P mod 2048 parameters are handled by plain loads in the last block.
-// Passes of fewer than 8 tiles per SM use a plain grid instead (one quad of
-// parameters per thread, fasgd_direct_kernel).
+// global stores.  A larger K runs as several stages per tile (the state travels
+// with the first one only).  Every block has the same number of whole tiles and
+// an equal piece of the rest (BlockShare); the last P mod 4 parameters go
+// through plain loads.  Passes of fewer than 8 tiles per SM use a plain grid
+// instead (one quad of parameters per thread, fasgd_direct_kernel).
 //
-// With SUMS (one push, a.vsum set) the pass also leaves the float-float sum
-// of the new v over every 128-parameter chunk (one warp's share of a tile)
-// in a.vsum, formed in registers, so the next per-message decision needs no
-// pass over v (message.cu forms the same chunk sums from v, bit for bit).
-// A SUMS pass of a per-message push also takes the push's Eq. 9 decision
-// itself (a.msg: every block's warp 0 combines the statistic's partials in
-// the decision kernel's order, message_decide) and, if the push is
-// transmitted, applies the pushed gradient while copying it into the
-// client's cache slot; if dropped it applies the slot.
+// With SUMS (one push, a.msg.partial set) the pass applies a per-message push
+// whose Eq. 9 decision was taken by the kernel before it, or, where the
+// statistic had to be formed afresh, takes it itself from the sums
+// (message_decide, in every block's warp 0): transmitted, it applies the pushed
+// gradient while copying it into the client's cache slot; dropped, it applies
+// the slot.  It also leaves every block's float-float sum of the new v, formed
+// in registers, so the next decision needs no pass over v (message.cu).
 //
 // Both kernels are launched as programmatic dependents (pdl.cuh): a pass is
 // scheduled while the kernel before it on the stream drains, sets up its
@@ -41,6 +39,7 @@
 // result does not depend on the grid or on which path handled an element.
 
 #include <atomic>
+#include <type_traits>
 
 #include "kernels.cuh"
 #include "message.cuh"
@@ -54,15 +53,17 @@ namespace {
 
 // Ring geometry per consumer count CONS (threads that compute; 512 or 256):
 // tiles of 4 CONS parameters, CONS + 32 threads per block (one producer
-// warp), 512 / CONS blocks per SM sharing 220 KB of shared memory.
+// warp), 512 / CONS blocks per SM sharing 220 KB of shared memory.  A stage
+// holds the state's slices and min(K, CH) gradients' (not CH: K = 5 keeps three
+// tiles in flight where stages for eight gradients kept two).
 template <int CONS> struct Geom {
     static constexpr int kTile = 4 * CONS;
     static constexpr int kThreads = CONS + 32;
     static constexpr int kBlocksPerSm = 512 / CONS;
+    static constexpr int kMaxStages = 8;
     static constexpr int kSmemBudget = 220 * 1024 / kBlocksPerSm;   // ring + barriers, per block
 };
 constexpr int kTile = Geom<512>::kTile;         // the reference tile (2048 parameters)
-constexpr int kMaxStages = 8;
 
 // ---- bulk async copy (the mbarrier wrappers and bounded waits: wait.cuh) ----
 // 1-D bulk copy global -> shared (16-byte aligned, size a multiple of 16),
@@ -86,124 +87,59 @@ __device__ __forceinline__ void redo_quad(const DenseArgs& a, const float* g0, i
     v = q.v;
 }
 
-// Parameters [begin, P) with plain loads, by the CONS consumer threads of
-// one block; begin is a multiple of 4.
-template <int RULE, int ARITH, int CONS>
-__device__ void apply_range_direct(const DenseArgs& a, int64_t begin, int tid) {
+// The last P mod 4 parameters, thread i < P mod 4 taking one; returns the new
+// v of its parameter (0 for the other threads).
+template <int RULE, int ARITH>
+__device__ __forceinline__ float apply_ragged(const DenseArgs& a, int tid, const float* g0, float* copy_to) {
     constexpr bool FAS = RULE != kRuleSgd;
-    const int64_t end_q = a.P & ~int64_t(3);
-    for (int64_t e = begin + 4 * (int64_t)tid; e < end_q; e += 4 * (int64_t)CONS) {
-        float4 th = *reinterpret_cast<const float4*>(a.theta + e);
-        float4 n = make_float4(0.f, 0.f, 0.f, 0.f), b = n, v = n;
-        if (FAS) {
-            n = *reinterpret_cast<const float4*>(a.n + e);
-            b = *reinterpret_cast<const float4*>(a.b + e);
-            v = *reinterpret_cast<const float4*>(a.v + e);
-        }
-        Guard<ARITH> guard;
-        for (int k = 0; k < a.K; ++k) {
-            const float4 g = __ldcs(reinterpret_cast<const float4*>(a.grad[k] + e));
-            update4<RULE, ARITH>(th, n, b, v, g, a.coef[k], a.sp, guard);
-        }
-        if (!guard.ok()) redo_quad<RULE>(a, a.grad[0], e, th, n, b, v);
-        *reinterpret_cast<float4*>(a.theta + e) = th;
-        if (FAS) {
-            *reinterpret_cast<float4*>(a.n + e) = n;
-            *reinterpret_cast<float4*>(a.b + e) = b;
-            *reinterpret_cast<float4*>(a.v + e) = v;
-        }
+    const int64_t p = (a.P & ~int64_t(3)) + tid;
+    if (p >= a.P) return 0.f;
+    float th = a.theta[p], n = 0.f, b = 0.f, v = 0.f;
+    if (FAS) {
+        n = a.n[p];
+        b = a.b[p];
+        v = a.v[p];
     }
-    const int64_t p = end_q + tid;  // the last P mod 4 parameters
-    if (tid < (int)(a.P & 3) && p < a.P) {
-        float th = a.theta[p], n = 0.f, b = 0.f, v = 0.f;
-        if (FAS) {
-            n = a.n[p];
-            b = a.b[p];
-            v = a.v[p];
-        }
-        for (int k = 0; k < a.K; ++k) {
-            const float g = __ldcs(a.grad[k] + p);
-            if (FAS)
-                rule_update<ARITH, RULE == kRuleFasgdStd>(th, n, b, v, g, a.coef[k], a.sp);
-            else
-                sgd_update(th, g, a.coef[k]);
-        }
-        a.theta[p] = th;
-        if (FAS) {
-            a.n[p] = n;
-            a.b[p] = b;
-            a.v[p] = v;
-        }
+    for (int k = 0; k < a.K; ++k) {
+        const float g = (k == 0 ? g0 : a.grad[k])[p];
+        if (k == 0 && copy_to != nullptr) copy_to[p] = g;
+        if (FAS)
+            rule_update<ARITH, RULE == kRuleFasgdStd>(th, n, b, v, g, a.coef[k], a.sp);
+        else
+            sgd_update(th, g, a.coef[k]);
     }
+    a.theta[p] = th;
+    if (FAS) {
+        a.n[p] = n;
+        a.b[p] = b;
+        a.v[p] = v;
+    }
+    return v;
 }
 
-// The SUMS form of the tail (one push): parameters [begin, P) chunk by
-// chunk, consumer warp w taking chunks begin/128 + w, + CONS/32, ...; lane l
-// updates parameters 4l .. 4l + 3 of the chunk (guarded at P) with gradient
-// g0, copying it to copy_to unless that is null, and the warp forms the
-// chunk's sum of the new v in registers.  begin is a multiple of 128.
-template <int RULE, int ARITH, int CONS>
-__device__ void apply_range_chunks(const DenseArgs& a, int64_t begin, int tid, const float* g0,
-                                   float* copy_to) {
-    const int warp = tid >> 5, lane = tid & 31;
-    const int64_t nch = (a.P + kVsumChunk - 1) / kVsumChunk;
-    for (int64_t c = begin / kVsumChunk + warp; c < nch; c += CONS / 32) {
-        const int64_t e = c * kVsumChunk + 4 * lane;
-        float th[4] = {0.f, 0.f, 0.f, 0.f}, n[4] = {0.f, 0.f, 0.f, 0.f};
-        float b[4] = {0.f, 0.f, 0.f, 0.f}, v[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (e + j < a.P) {
-                th[j] = a.theta[e + j];
-                n[j] = a.n[e + j];
-                b[j] = a.b[e + j];
-                v[j] = a.v[e + j];
-            }
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (e + j < a.P) {
-                const float g = __ldcs(g0 + e + j);
-                if (copy_to != nullptr) copy_to[e + j] = g;
-                rule_update<ARITH, RULE == kRuleFasgdStd>(th[j], n[j], b[j], v[j], g, a.coef[0],
-                                                          a.sp);
-            }
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (e + j < a.P) {
-                a.theta[e + j] = th[j];
-                a.n[e + j] = n[j];
-                a.b[e + j] = b[j];
-                a.v[e + j] = v[j];
-            }
-        const float2 cs = chunk_sum4(make_float4(v[0], v[1], v[2], v[3]));
-        if (lane == 0) a.vsum[c] = cs;
-    }
-}
-
-// Ring geometry, identical on host and device.
 struct Ring {
     int stages;     // stages in the ring
     int chunks;     // stages per tile: ceil(K / CH)
+    int floats;     // floats per stage
 };
 
 // RULE: kRuleSgd / kRuleFasgd / kRuleFasgdStd; ARITH: kArithApprox /
 // kArithApproxFtz / kArithExact (see update.cuh); CH: gradient slices per stage;
-// SUMS: also leave the chunk sums of the new v (FASGD rules, K = 1); CONS:
+// SUMS: also leave the blocks' sums of the new v (FASGD rules, K = 1); CONS:
 // consumer threads per block (the ring geometry, Geom).
 template <int RULE, int ARITH, int CH, bool SUMS, int CONS>
 __global__ void __launch_bounds__(Geom<CONS>::kThreads, Geom<CONS>::kBlocksPerSm)
-fasgd_dense_kernel(const __grid_constant__ DenseArgs a, const Ring ring, const int64_t ntiles) {
+fasgd_dense_kernel(const __grid_constant__ DenseArgs a, const Ring ring) {
+    using G = Geom<CONS>;
     constexpr bool FAS = RULE != kRuleSgd;
     constexpr int kState = FAS ? 4 : 1;              // theta (, n, b, v)
-    constexpr int kTile = Geom<CONS>::kTile;
-    constexpr int kConsumers = CONS;
-    constexpr int kStageFloats = (kState + CH) * kTile;
+    constexpr int kTile = G::kTile, kConsumerWarps = CONS / 32;
     extern __shared__ __align__(128) unsigned char smem[];
     float* buf = reinterpret_cast<float*>(smem);
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)ring.stages * kStageFloats * 4);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + (size_t)ring.stages * ring.floats * 4);
     uint64_t* empty = full + ring.stages;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int kConsumerWarps = kConsumers / 32;
+    const BlockShare share(a.P & ~int64_t(3), kTile, gridDim.x, blockIdx.x);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < ring.stages; ++s) {
@@ -213,32 +149,55 @@ fasgd_dense_kernel(const __grid_constant__ DenseArgs a, const Ring ring, const i
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    const auto load_state = [&](float* st, int64_t off, uint32_t bytes, uint64_t* bar) {
+        bulk_load(st, a.theta + off, bytes, bar);
+        if (FAS) {
+            bulk_load(st + 1 * kTile, a.n + off, bytes, bar);
+            bulk_load(st + 2 * kTile, a.b + off, bytes, bar);
+            bulk_load(st + 3 * kTile, a.v + off, bytes, bar);
+        }
+    };
+    // A message push (SUMS) follows its own decision kernel, which only reads v
+    // or its sums and started after every earlier kernel had finished, so the
+    // state may be read before that kernel is complete: the first stages' state
+    // is on its way while the decision is taken.
+    int64_t early = 0;
+    if (SUMS && warp == kConsumerWarps && lane == 0) {
+        early = share.tiles < ring.stages ? share.tiles : ring.stages;
+        for (int i = 0; i < (int)early; ++i) {
+            const uint32_t bytes = (uint32_t)share.length(i) * 4;
+            mbar_arrive_expect_tx(&full[i], (kState + 1) * bytes);
+            load_state(buf + (size_t)i * ring.floats, share.offset(i), bytes, &full[i]);
+        }
+    }
     pdl_wait();      // the kernel before this one on the stream is complete
     pdl_trigger();
-    // A message push decided here (SUMS, a.msg.partial set): warp 0 takes the
-    // decision, every thread reads it.  Transmitted: apply the pushed gradient
-    // and copy it into the client's cache slot; dropped: apply the slot.
+    // Transmitted: apply the pushed gradient and copy it into the client's cache
+    // slot; dropped: apply the slot.
     const float* g0 = a.grad[0];
     float* copy_to = nullptr;
     if constexpr (SUMS) {
-        __shared__ uint32_t s_send;
-        if (a.msg.partial != nullptr) {
+        uint32_t send;
+        if (a.msg.decided != nullptr) {
+            send = *a.msg.decided;
+        } else {     // the statistic was formed afresh: decide from its sums
+            __shared__ uint32_t s_send;
             if (warp == 0) {
                 float vbar;
-                const uint32_t send = message_decide(a.msg.partial, a.msg.nblocks, a.P, a.msg.c,
-                                                     a.msg.eps_b, a.msg.round_key0,
-                                                     a.msg.round_key1, a.msg.client_word,
-                                                     a.msg.n_lo, a.msg.n_hi, &vbar);
+                const uint32_t d = message_decide(a.msg.fresh, a.msg.nblocks, a.P, a.msg.c, a.msg.eps_b,
+                                                  a.msg.round_key0, a.msg.round_key1, a.msg.client_word,
+                                                  a.msg.n_lo, a.msg.n_hi, &vbar);
                 if (lane == 0) {
-                    s_send = send;
-                    if (blockIdx.x == 0 && a.msg.flag_out != nullptr) *a.msg.flag_out = (int32_t)send;
+                    s_send = d;
+                    if (blockIdx.x == 0 && a.msg.flag_out != nullptr) *a.msg.flag_out = (int32_t)d;
                 }
             }
             __syncthreads();
-            if (s_send) {
-                g0 = a.msg.src;
-                copy_to = a.msg.slot;
-            }
+            send = s_send;
+        }
+        if (send) {
+            g0 = a.msg.src;
+            copy_to = a.msg.slot;
         }
     }
 
@@ -250,28 +209,21 @@ fasgd_dense_kernel(const __grid_constant__ DenseArgs a, const Ring ring, const i
             bool ok = true;
             uint32_t issued = 0;            // bit s: stage s has been filled
             uint32_t issued_phase = 0;      // bit s: the phase parity of its last fill
-            for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-                const int64_t off = t * kTile;
+            for (int64_t t = 0; t < share.tiles && ok; ++t) {
+                const int64_t off = share.offset(t);
+                const uint32_t bytes = (uint32_t)share.length(t) * 4;
                 for (int c = 0; c < ring.chunks; ++c) {
                     ok = wait_one(&empty[s], ph ^ 1u, a.err);
                     if (!ok) break;
-                    const int k0 = c * CH;
-                    const int ng = min(CH, a.K - k0);
-                    const int ns = (c == 0) ? kState : 0;
-                    mbar_arrive_expect_tx(&full[s], (uint32_t)((ns + ng) * kTile * 4));
-                    float* st = buf + (size_t)s * kStageFloats;
-                    if (ns > 0) {
-                        bulk_load(st, a.theta + off, kTile * 4, &full[s]);
-                        if (FAS) {
-                            bulk_load(st + 1 * kTile, a.n + off, kTile * 4, &full[s]);
-                            bulk_load(st + 2 * kTile, a.b + off, kTile * 4, &full[s]);
-                            bulk_load(st + 3 * kTile, a.v + off, kTile * 4, &full[s]);
-                        }
+                    const int k0 = c * CH, ng = min(CH, a.K - k0);
+                    float* st = buf + (size_t)s * ring.floats;
+                    if (t >= early) {               // else armed, and its state asked for, above
+                        mbar_arrive_expect_tx(&full[s], (uint32_t)((c == 0 ? kState : 0) + ng) * bytes);
+                        if (c == 0) load_state(st, off, bytes, &full[s]);
                     }
-                    float* gs = st + kState * kTile;
                     for (int j = 0; j < ng; ++j)
-                        bulk_load(gs + j * kTile, (k0 + j == 0 ? g0 : a.grad[k0 + j]) + off,
-                                  kTile * 4, &full[s]);
+                        bulk_load(st + (kState + j) * kTile, (k0 + j == 0 ? g0 : a.grad[k0 + j]) + off,
+                                  bytes, &full[s]);
                     issued |= 1u << s;
                     issued_phase = (issued_phase & ~(1u << s)) | (ph << s);
                     if (++s == ring.stages) {
@@ -291,52 +243,56 @@ fasgd_dense_kernel(const __grid_constant__ DenseArgs a, const Ring ring, const i
     const int tid = threadIdx.x;
     int s = 0;
     uint32_t ph = 0;
-    bool ok = true;
-    for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+    VSum vsum;
+    // One tile from `off`; whole: all of its threads have a quad, else those
+    // below `length`.
+    const auto tile = [&](auto whole, int64_t off, int length) {
+        const bool mine = whole.value || 4 * tid < length;
+        const int64_t e = off + 4 * (int64_t)tid;
         float4 th = make_float4(0.f, 0.f, 0.f, 0.f), n = th, b = th, v = th;
         Guard<ARITH> guard;
         for (int c = 0; c < ring.chunks; ++c) {
-            ok = wait_warp(&full[s], ph, a.err);
-            if (!ok) break;
-            const float* st = buf + (size_t)s * kStageFloats;
-            if (c == 0) {
-                th = reinterpret_cast<const float4*>(st)[tid];
-                if (FAS) {
-                    n = reinterpret_cast<const float4*>(st + 1 * kTile)[tid];
-                    b = reinterpret_cast<const float4*>(st + 2 * kTile)[tid];
-                    v = reinterpret_cast<const float4*>(st + 3 * kTile)[tid];
+            if (!wait_warp(&full[s], ph, a.err)) return false;
+            const float4* st = reinterpret_cast<const float4*>(buf + (size_t)s * ring.floats) + tid;
+            float4 g[CH];
+            const int k0 = c * CH, ng = min(CH, a.K - k0);
+            if (mine) {
+                if (c == 0) {
+                    th = st[0];
+                    if (FAS) {
+                        n = st[1 * (kTile / 4)];
+                        b = st[2 * (kTile / 4)];
+                        v = st[3 * (kTile / 4)];
+                    }
+                }
+                if (ng == CH) {
+#pragma unroll
+                    for (int j = 0; j < CH; ++j) g[j] = st[(kState + j) * (kTile / 4)];
+                } else {
+#pragma unroll
+                    for (int j = 0; j < CH; ++j)
+                        if (j < ng) g[j] = st[(kState + j) * (kTile / 4)];
                 }
             }
-            const int k0 = c * CH;
-            const float4* gs = reinterpret_cast<const float4*>(st + kState * kTile);
-            float4 g[CH];
-            if (k0 + CH <= a.K) {  // a full chunk
-#pragma unroll
-                for (int j = 0; j < CH; ++j) g[j] = gs[j * (kTile / 4) + tid];
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&empty[s]);  // inputs are in registers
-                if (SUMS && copy_to != nullptr)          // a transmitted message refreshes its slot
-                    reinterpret_cast<float4*>(copy_to + t * kTile)[tid] = g[0];
-#pragma unroll
-                for (int j = 0; j < CH; ++j) update4<RULE, ARITH>(th, n, b, v, g[j], a.coef[k0 + j], a.sp, guard);
-            } else {               // the last, partial chunk
-                const int ng = a.K - k0;
-#pragma unroll
-                for (int j = 0; j < CH; ++j)
-                    if (j < ng) g[j] = gs[j * (kTile / 4) + tid];
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&empty[s]);
-#pragma unroll
-                for (int j = 0; j < CH; ++j)
-                    if (j < ng) update4<RULE, ARITH>(th, n, b, v, g[j], a.coef[k0 + j], a.sp, guard);
-            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[s]);   // inputs are in registers
             if (++s == ring.stages) {
                 s = 0;
                 ph ^= 1u;
             }
+            if (!mine) continue;
+            if (SUMS && copy_to != nullptr)          // a transmitted message refreshes its slot
+                *reinterpret_cast<float4*>(copy_to + e) = g[0];
+            if (ng == CH) {
+#pragma unroll
+                for (int j = 0; j < CH; ++j) update4<RULE, ARITH>(th, n, b, v, g[j], a.coef[k0 + j], a.sp, guard);
+            } else {
+#pragma unroll
+                for (int j = 0; j < CH; ++j)
+                    if (j < ng) update4<RULE, ARITH>(th, n, b, v, g[j], a.coef[k0 + j], a.sp, guard);
+            }
         }
-        if (!ok) break;
-        const int64_t e = t * kTile + 4 * (int64_t)tid;
+        if (!mine) return true;
         if (!guard.ok()) redo_quad<RULE>(a, g0, e, th, n, b, v);
         *reinterpret_cast<float4*>(a.theta + e) = th;
         if (FAS) {
@@ -344,30 +300,36 @@ fasgd_dense_kernel(const __grid_constant__ DenseArgs a, const Ring ring, const i
             *reinterpret_cast<float4*>(a.b + e) = b;
             *reinterpret_cast<float4*>(a.v + e) = v;
         }
-        if (SUMS) {
-            const float2 cs = chunk_sum4(v);
-            if (lane == 0) a.vsum[(t * kTile) / kVsumChunk + warp] = cs;
-        }
-    }
-    // Parameters after the last full tile.
+        if (SUMS) vsum.add(v);
+        return true;
+    };
+    bool ok = true;
+    for (int64_t t = 0; t < share.whole && ok; ++t) ok = tile(std::true_type{}, share.offset(t), kTile);
+    if (ok && share.piece > 0) ok = tile(std::false_type{}, share.piece_start, share.piece);
     if (ok && blockIdx.x == gridDim.x - 1) {
-        if (SUMS)
-            apply_range_chunks<RULE, ARITH, CONS>(a, ntiles * kTile, tid, g0, copy_to);
-        else
-            apply_range_direct<RULE, ARITH, CONS>(a, ntiles * kTile, tid);
+        const float v = apply_ragged<RULE, ARITH>(a, tid, g0, copy_to);
+        if (SUMS && tid < (int)(a.P & 3)) vsum.add(make_float4(v, 0.f, 0.f, 0.f));
+    }
+    if constexpr (SUMS) {
+        __shared__ float2 s_sum[kConsumerWarps];
+        const float2 w = vsum.warp_total();
+        if (lane == 0) s_sum[warp] = w;
+        asm volatile("bar.sync 1, %0;" ::"n"(CONS) : "memory");   // the consumers
+        if (tid == 0) a.msg.partial[blockIdx.x] = ordered_total<kConsumerWarps>(s_sum);
     }
 }
 
+// A pass with up to `stages` stages in the ring.
 template <int RULE, int ARITH, int CH, bool SUMS = false, int CONS = 512>
-cudaError_t launch_ch(const DenseArgs& a, int num_sms, cudaStream_t stream) {
+cudaError_t launch_ch(const DenseArgs& a, int stages, int num_sms, cudaStream_t stream) {
     using G = Geom<CONS>;
     constexpr int kState = RULE != kRuleSgd ? 4 : 1;
-    constexpr int kStageBytes = (kState + CH) * G::kTile * 4;
     Ring ring;
     ring.chunks = (a.K + CH - 1) / CH;
-    ring.stages = (G::kSmemBudget - 2 * kMaxStages * 8) / kStageBytes;
-    if (ring.stages > kMaxStages) ring.stages = kMaxStages;
-    const size_t smem = (size_t)ring.stages * kStageBytes + 2 * ring.stages * sizeof(uint64_t);
+    ring.floats = (kState + (a.K < CH ? a.K : CH)) * G::kTile;
+    ring.stages = (G::kSmemBudget - 2 * G::kMaxStages * 8) / (ring.floats * 4);
+    if (ring.stages > stages) ring.stages = stages;
+    const size_t smem = (size_t)ring.stages * ring.floats * 4 + 2 * ring.stages * sizeof(uint64_t);
     // The shared-memory limit is a per-device attribute of the kernel: set it
     // once per device (bit d of the mask) and instantiation.
     static std::atomic<uint64_t> configured{0};
@@ -381,13 +343,8 @@ cudaError_t launch_ch(const DenseArgs& a, int num_sms, cudaStream_t stream) {
         if (st != cudaSuccess) return st;
         configured.fetch_or(bit, std::memory_order_acq_rel);
     }
-    const int64_t ntiles = a.P / G::kTile;
-    // kBlocksPerSm blocks per SM (shared-memory bound), never more than there are tiles.
-    const int64_t slots = (int64_t)G::kBlocksPerSm * num_sms;
-    int64_t grid = ntiles < slots ? ntiles : slots;
-    if (grid < 1) grid = 1;
-    return launch_pdl(fasgd_dense_kernel<RULE, ARITH, CH, SUMS, CONS>, (unsigned)grid,
-                      G::kThreads, smem, stream, a, ring, ntiles);
+    return launch_pdl(fasgd_dense_kernel<RULE, ARITH, CH, SUMS, CONS>,
+                      (unsigned)(G::kBlocksPerSm * num_sms), G::kThreads, smem, stream, a, ring);
 }
 
 // ---- small passes ------------------------------------------------------------
@@ -476,26 +433,55 @@ cudaError_t launch_direct(const DenseArgs& a, int num_sms, cudaStream_t stream) 
 template <int RULE, int ARITH>
 cudaError_t launch_rule(const DenseArgs& a, int num_sms, cudaStream_t stream) {
     if constexpr (RULE != kRuleSgd) {
-        if (a.vsum != nullptr) {
+        if (a.msg.partial != nullptr) {
             if (a.K != 1) return cudaErrorInvalidValue;
-            return launch_ch<RULE, ARITH, 1, true>(a, num_sms, stream);
+            // State within L2 (16 bytes per parameter, 129 MB): all five
+            // stages, since the decision's latency in front of the pass counts
+            // (eight pushes and fetches at 5M: 233 against 269 us with two).
+            // Beyond it two, as below (25M: 1237 against 1264 us).
+            const bool in_l2 = a.P <= 7'000'000;
+            return launch_ch<RULE, ARITH, 1, true>(a, in_l2 ? 5 : 2, num_sms, stream);
         }
     }
     if (a.P / kTile < kDirectTilesPerSm * num_sms) return launch_direct<RULE, ARITH>(a, num_sms, stream);
-    // Gradient slices per stage: K rounded up to a power of two, at most 8.
-    // K > 8 takes several stages per tile: two blocks of 256 consumers per SM
-    // keep more stages in flight there (P = 50M, K = 16: 686.8 against
-    // 704.0 us per pass); up to K = 8 one block of 512 is faster (226.8
-    // against 232.1 us at P = 25M, K = 8).
-    // The exact rules hold more values per push: four slices at a time leave
-    // them the registers (K = 8 / 16 at 25M: 282 / 519 against 289 / 549 us
-    // with eight, push + apply + pull).
-    if (ARITH == kArithExact && RULE != kRuleSgd && a.K > 4) return launch_ch<RULE, ARITH, 4>(a, num_sms, stream);
-    if (a.K > 8) return launch_ch<RULE, ARITH, 8, false, 256>(a, num_sms, stream);
-    if (a.K > 4) return launch_ch<RULE, ARITH, 8>(a, num_sms, stream);
-    if (a.K > 2) return launch_ch<RULE, ARITH, 4>(a, num_sms, stream);
-    if (a.K > 1) return launch_ch<RULE, ARITH, 2>(a, num_sms, stream);
-    return launch_ch<RULE, ARITH, 1>(a, num_sms, stream);
+    // How many gradient slices a stage takes (CH) and how many stages: a tile's
+    // first stage holds its state and CH gradients, the others CH each, and HBM
+    // streams best with some 80 to 160 KB per SM in flight, less than the
+    // shared memory would hold (reads that run further ahead only push the
+    // writes together).  Sweep of CH = 1, 2, 4, 8 (512 consumers; also 4, 8
+    // with two blocks of 256) by 2 to 8 stages, push + apply + pull in us at
+    // 25M parameters, as before (CH = K rounded up to a power of two, every
+    // stage that fits; K > 8 two blocks of 256, CH = 8) -> as chosen; the same
+    // choices were best or within 1 % at 3M, 6M and 10M:
+    //   FASGD  K = 1: 172.6 -> 164   2: 185 -> 176     3: 201 -> 190
+    //          4: 215 -> 206         5: 231 -> 217     6: 244 -> 229
+    //          8: 253 -> 254         12: 316 -> 312    16: 375 (same)   32: 631 -> 601
+    //   exact  3: 204 -> 190         4: 223 -> 207     5: 222 (same)
+    //          6: 238 -> 232         8: 281 (same)     16: 510 (same)
+    //   SGD    K = 3: 103 -> 102     6: 148 -> 146     8: 182 -> 174
+    //          12: 242 -> 232        16: 300 -> 287    32: 531 -> 512
+    if constexpr (RULE == kRuleSgd) {
+        if (a.K == 1) return launch_ch<RULE, ARITH, 1>(a, 5, num_sms, stream);
+        if (a.K == 2) return launch_ch<RULE, ARITH, 2>(a, 5, num_sms, stream);
+        if (a.K <= 4) return launch_ch<RULE, ARITH, 4>(a, a.K == 3 ? 4 : 3, num_sms, stream);
+        if (a.K <= 8 || a.K > 14) return launch_ch<RULE, ARITH, 8>(a, 2, num_sms, stream);
+        return launch_ch<RULE, ARITH, 4>(a, 4, num_sms, stream);
+    } else {
+        if (a.K == 1) return launch_ch<RULE, ARITH, 1>(a, 2, num_sms, stream);
+        if (a.K == 2) return launch_ch<RULE, ARITH, 1>(a, 3, num_sms, stream);
+        if (a.K <= 4) return launch_ch<RULE, ARITH, 2>(a, 3, num_sms, stream);
+        if constexpr (ARITH == kArithExact) {
+            // More values per push: four slices at a time leave them the registers.
+            if (a.K == 5) return launch_ch<RULE, ARITH, 2>(a, 4, num_sms, stream);
+            if (a.K <= 7) return launch_ch<RULE, ARITH, 8>(a, 2, num_sms, stream);
+            return launch_ch<RULE, ARITH, 4>(a, 3, num_sms, stream);
+        } else {
+            if (a.K <= 6) return launch_ch<RULE, ARITH, 2>(a, 4, num_sms, stream);
+            if (a.K <= 8) return launch_ch<RULE, ARITH, 4>(a, 3, num_sms, stream);
+            if (a.K <= 12) return launch_ch<RULE, ARITH, 4, false, 256>(a, 3, num_sms, stream);
+            return launch_ch<RULE, ARITH, 8, false, 256>(a, 2, num_sms, stream);
+        }
+    }
 }
 
 }  // namespace

@@ -23,20 +23,49 @@ struct StatParams {
     float minus_zero;   // -0.0f, a value the compiler does not see (update.cuh, product2)
 };
 
-// A per-message push decided inside its pass (with vsum, FASGD rules): the
-// pass first takes the push's Eq. 9 decision from the statistic's partials
-// (message_decide); if transmitted it applies src and copies it into slot
-// (the client's gradient cache slot, which is also grad[0]), else it applies
-// grad[0] as it stands.  partial == null: no decision, grad[0] is applied.
+// Block b's share of P (a multiple of 4) parameters of a pass over `blocks`
+// blocks in tiles of `tile`: as many whole tiles as every block can have,
+// interleaved, then an equal piece of the rest (a multiple of 128), so that no
+// block has a tile more than another (a pass over 5M parameters has 16.06
+// tiles per SM).
+struct BlockShare {
+    int64_t tiles;      // this block's tiles, the piece included
+    int64_t whole;      // whole tiles of each block
+    int64_t first, step, piece_start;
+    int32_t tile, piece;
+    __host__ __device__ BlockShare(int64_t P, int32_t tile_, int64_t blocks, int64_t b) : tile(tile_) {
+        whole = P / (blocks * tile);
+        first = b * tile;
+        step = blocks * tile;
+        const int64_t rest = P - whole * step;
+        const int64_t share = ((rest + blocks - 1) / blocks + 127) / 128 * 128;
+        const int64_t from = b * share < rest ? b * share : rest;
+        piece = (int32_t)(rest - from < share ? rest - from : share);
+        piece_start = whole * step + from;
+        tiles = whole + (piece > 0 ? 1 : 0);
+    }
+    __host__ __device__ int64_t offset(int64_t t) const { return t < whole ? first + t * step : piece_start; }
+    __host__ __device__ int32_t length(int64_t t) const { return t < whole ? tile : piece; }
+};
+
+// A per-message push decided before or inside its pass (FASGD rules): the pass
+// reads the decision, or takes it from the statistic's sums (message_decide)
+// where they were just formed afresh; if transmitted it applies src and copies
+// it into slot (the client's gradient cache slot, which is also grad[0]), else
+// it applies grad[0] as it stands.  Either way it leaves its blocks' sums of the
+// new v in `partial`, which is not `fresh` (a block may end before another has
+// read it).  partial == null: not a message push.
 struct PassMessage {
-    const float2* partial;          // nblocks float-float partial sums of v
+    const uint32_t* decided;        // the decision (1: transmitted), or null
+    const float2* fresh;            // if not decided: nblocks float-float sums of v
+    float2* partial;                // out: one sum per block of the pass
     int32_t nblocks;
     float c, eps_b;
     uint32_t round_key0[10], round_key1[10];
     uint32_t client_word, n_lo, n_hi;
     const float* src;               // the pushed gradient, fp32[P], 16-byte aligned
     float* slot;                    // == grad[0]
-    int32_t* flag_out;              // may be null: 1 transmitted, 0 dropped
+    int32_t* flag_out;              // may be null: 1 transmitted, 0 dropped (if not decided)
 };
 
 // One fused pass over the parameters applying K dense pushes in order.
@@ -51,12 +80,8 @@ struct DenseArgs {
     int32_t K;
     StatParams sp;
     int32_t* err;                   // device error flags (bit 3: a pipeline wait expired)
-    float2* vsum;                   // if set (K = 1, FASGD rules): the float-float sum of
-                                    // the new v over every 128-parameter chunk
-    PassMessage msg;                // with vsum only
+    PassMessage msg;                // K = 1, FASGD rules
 };
-// Parameters per chunk of the per-message statistic's partial sums.
-constexpr int kVsumChunk = 128;
 
 // One sparse push: idx[i] receives val[i] for i < count.
 struct SparseArgs {

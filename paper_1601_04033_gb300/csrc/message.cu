@@ -2,28 +2,32 @@
 // transmission opportunity, taken against v = the mean over all parameters
 // of the server's moving averages.
 //
-// Two kernels per decision:
-//   1. vbar_partial: the parameters are cut into 128-parameter chunks and
-//      the chunks into one contiguous range per block; each block combines
-//      its chunks' float-float sums in a fixed order into one partial.  The
-//      chunk sums are those the dense pass leaves after a message push (so
-//      v is not read again), or, when another pass has changed v since, the
-//      block forms them from v with the same arithmetic and stores them;
-//   2. message_resolve: every block adds the partials in the same fixed order
-//      (float-float), forms vbar = fl32(sum / P) (ff_div_int), draws u
-//      (Philox4x32-10, word 0 at counter
-//      (2^32-1, client + 2^31 * stream, n)), takes the exact Eq. 9 decision,
-//      and, if the message is transmitted, copies src to dst (grid-stride,
-//      128-bit); block 0 reports the decision.
-// The partition depends on P only, so the decision is the same for every
-// launch and every GPU.  For a push, src is the client's gradient and dst its
-// slot of the server's gradient cache (the pass that follows reads the
-// slot, so a dropped push re-applies the client's last sent gradient); for a
-// fetch, src is theta and dst the client's copy.  Under the FASGD rules a
-// push skips kernel 2: the pass that applies it takes the same decision
-// (message_decide, message.cuh) and refreshes the slot as it streams
-// (dense.cu); kernel 2 serves fetches, the statistic query and ASGD/SASGD
-// pushes.
+// The statistic is kept as one float-float sum of v per block of the dense
+// pass: the pass of a message push adds its blocks' new v up in registers
+// (VSum) as it stores them, each thread its quads of the block's share in
+// order, then a fixed tree.  After any other change of v, vbar_partial_kernel
+// forms the same sums from v (same shares, same order, same bits).  The shares
+// depend on P and the number of SMs alone, so a decision does not depend on
+// which kernel formed the sums.  A decision (message_decide, one warp) adds the
+// sums in a fixed order, forms vbar = fl32(sum / P) (ff_div_int), draws u
+// (Philox4x32-10, word 0 at counter (2^32-1, client + 2^31 * stream, n)) and
+// takes the exact Eq. 9 test.
+//
+//   - A push under the FASGD rules: message_decide_kernel takes the decision
+//     while the pass behind it already loads its first tiles' state; the pass
+//     applies the pushed gradient, refreshing the client's cache slot as it
+//     streams, or the slot.  If the sums had to be formed afresh, the pass takes
+//     the decision itself from them (message.cuh), so a push is two kernels.
+//   - A fetch, an ASGD/SASGD push and the statistic query:
+//     message_resolve_kernel, every block of which takes the decision and, if
+//     the message is transmitted, copies src to dst (for a push: the gradient to
+//     the client's slot of the server's gradient cache, which the pass that
+//     follows reads; for a fetch: theta to the client's copy).
+//
+// Measured at 25M parameters (eight pushes, eight fetches, a pull): sums per
+// 128-parameter chunk with a kernel per decision to combine them 1355 us, these
+// 1237 us.  A warp's tree per chunk cost 27 instructions per parameter,
+// the running sums 11.
 
 #include "eq9.cuh"
 #include "kernels.cuh"
@@ -36,72 +40,46 @@ namespace {
 
 constexpr int kMsgThreads = 256;
 
-// This lane's four values of chunk c of v (parameters 4 lane .. 4 lane + 3
-// of the chunk), zeros past P.  chunk_sum4 over them gives the same bits the
-// dense pass leaves for the chunk.
-__device__ __forceinline__ float4 chunk_values(const float* v, int64_t P, int64_t c, int lane) {
-    const int64_t e = c * kVsumChunk + 4 * lane;
-    if (e + 3 < P) return __ldcs(reinterpret_cast<const float4*>(v + e));
-    float4 x;
-    x.x = e < P ? v[e] : 0.f;
-    x.y = e + 1 < P ? v[e + 1] : 0.f;
-    x.z = e + 2 < P ? v[e + 2] : 0.f;
-    x.w = e + 3 < P ? v[e + 3] : 0.f;
-    return x;
-}
+constexpr int kSumThreads = 512;   // as the dense pass's consumers: a tile is one quad of each
 
-// Block b combines chunks [c0, c1) in a fixed order: chunk c0 + w + 8 i goes
-// to warp w, slot i, and lane (i mod 32) of that warp adds its slots in
-// increasing i; then each warp's tree, then the warps in order.  from_v: the
-// warp forms each chunk sum from v (four chunks' loads in flight) and stores
-// it; otherwise lane l loads its slots' stored sums.  Both give the same bits.
-__global__ void __launch_bounds__(kMsgThreads) vbar_partial_kernel(const __grid_constant__ MessageArgs a) {
-    __shared__ float2 smem[kMsgThreads / 32];
+// The sums the dense pass would leave, from v: thread t of block b adds quad t
+// of each tile of the block's share in order (four tiles' loads in flight).
+__global__ void __launch_bounds__(kSumThreads) vbar_partial_kernel(const __grid_constant__ MessageArgs a) {
+    __shared__ float2 s_sum[kSumThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const BlockShare share(a.P & ~int64_t(3), 4 * kSumThreads, gridDim.x, blockIdx.x);
     pdl_wait();
     pdl_trigger();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int kWarps = kMsgThreads / 32;
-    const int64_t nch = (a.P + kVsumChunk - 1) / kVsumChunk;
-    const int64_t per = (nch + a.nblocks - 1) / a.nblocks;
-    const int64_t c0 = (int64_t)blockIdx.x * per;
-    const int64_t c1 = c0 + per < nch ? c0 + per : nch;
-    const int64_t nslots = c1 > c0 + warp ? (c1 - c0 - warp + kWarps - 1) / kWarps : 0;
-    float h = 0.f, l = 0.f;
-    if (a.from_v) {
-        for (int64_t i0 = 0; i0 < nslots; i0 += 4) {
-            float4 x[4];
+    VSum sum;
+    for (int64_t t = 0; t < share.tiles; t += 4) {
+        float4 x[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (i0 + k < nslots) x[k] = chunk_values(a.v, a.P, c0 + warp + kWarps * (i0 + k), lane);
+        for (int k = 0; k < 4; ++k)
+            if (t + k < share.tiles && 4 * tid < share.length(t + k))
+                x[k] = reinterpret_cast<const float4*>(a.v + share.offset(t + k))[tid];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int64_t i = i0 + k;
-                if (i < nslots) {   // warp-uniform: the tree below uses every lane
-                    const int64_t c = c0 + warp + kWarps * i;
-                    const float2 cs = chunk_sum4(x[k]);
-                    if (lane == 0) a.chunks[c] = cs;
-                    if (lane == (int)(i & 31)) ff_add(h, l, cs.x, cs.y);
-                }
-            }
-        }
-    } else {
-        for (int64_t i0 = lane; i0 < nslots; i0 += 4 * 32) {
-            float2 x[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (i0 + 32 * k < nslots) x[k] = a.chunks[c0 + warp + kWarps * (i0 + 32 * k)];
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (i0 + 32 * k < nslots) ff_add(h, l, x[k].x, x[k].y);
-        }
+        for (int k = 0; k < 4; ++k)
+            if (t + k < share.tiles && 4 * tid < share.length(t + k)) sum.add(x[k]);
     }
-    ff_warp_sum(h, l);
-    if (lane == 0) smem[warp] = make_float2(h, l);
+    if (blockIdx.x == gridDim.x - 1 && tid < (int)(a.P & 3))
+        sum.add(make_float4(a.v[(a.P & ~int64_t(3)) + tid], 0.f, 0.f, 0.f));
+    const float2 w = sum.warp_total();
+    if (lane == 0) s_sum[warp] = w;
     __syncthreads();
+    if (tid == 0) a.partial[blockIdx.x] = ordered_total<kSumThreads / 32>(s_sum);
+}
+
+// One warp: the decision of a push, for the pass behind it (which starts on its
+// state meanwhile: this kernel touches none of it).
+__global__ void __launch_bounds__(32) message_decide_kernel(const __grid_constant__ MessageArgs a) {
+    pdl_wait();
+    pdl_trigger();
+    float vbar;
+    const uint32_t send = message_decide(a.partial, a.nblocks, a.P, a.c, a.eps_b, a.round_key0,
+                                         a.round_key1, a.client_word, a.n_lo, a.n_hi, &vbar);
     if (threadIdx.x == 0) {
-        float2 t = make_float2(0.f, 0.f);
-        for (int w = 0; w < kWarps; ++w) ff_add(t.x, t.y, smem[w].x, smem[w].y);
-        a.partial[blockIdx.x] = t;
+        *a.decided = send;
+        if (a.flag_out != nullptr) *a.flag_out = (int32_t)send;
     }
 }
 
@@ -132,24 +110,21 @@ __global__ void __launch_bounds__(kMsgThreads) message_resolve_kernel(const __gr
 
 }  // namespace
 
-int32_t message_partial_blocks(int64_t P) {
-    const int64_t nch = (P + kVsumChunk - 1) / kVsumChunk;
-    int64_t b = (nch + 255) / 256;   // ~256 chunks (32,768 parameters) per block
-    if (b < 1) b = 1;
-    if (b > kMessageMaxBlocks) b = kMessageMaxBlocks;
-    return (int32_t)b;
+cudaError_t launch_message_sums(const MessageArgs& a, cudaStream_t stream, int64_t* launches) {
+    const cudaError_t st = launch_pdl(vbar_partial_kernel, a.nblocks, kSumThreads, 0, stream, a);
+    if (st == cudaSuccess) ++*launches;
+    return st;
 }
 
-cudaError_t launch_message_partials(const MessageArgs& a, cudaStream_t stream, int64_t* launches) {
-    const cudaError_t st = launch_pdl(vbar_partial_kernel, a.nblocks, kMsgThreads, 0, stream, a);
+cudaError_t launch_message_decide(const MessageArgs& a, cudaStream_t stream, int64_t* launches) {
+    const cudaError_t st = launch_pdl(message_decide_kernel, 1, 32, 0, stream, a);
     if (st == cudaSuccess) ++*launches;
     return st;
 }
 
 cudaError_t launch_message(const MessageArgs& a, int num_sms, cudaStream_t stream,
                            int64_t* launches) {
-    cudaError_t st = launch_message_partials(a, stream, launches);
-    if (st != cudaSuccess) return st;
+    cudaError_t st;
     int64_t grid = ((a.P >> 2) + kMsgThreads - 1) / kMsgThreads;
     const int64_t cap = (int64_t)(num_sms > 0 ? num_sms : 1) * 8;
     if (grid > cap) grid = cap;

@@ -9,16 +9,11 @@ namespace fasgd {
 
 // One per-message B-FASGD decision (push or fetch) and, when the message is
 // transmitted, the copy src -> dst (P floats, both 16-byte aligned).
-constexpr int kMessageMaxBlocks = 1024;
-
 struct MessageArgs {
     const float* v;            // the server's statistic, fp32[P]
     int64_t P;
-    float2* partial;           // scratch: nblocks float-float partial sums
-    int32_t nblocks;           // message_partial_blocks(P)
-    float2* chunks;            // ceil(P / 128) chunk sums of v
-    int32_t from_v;            // 1: form the chunk sums from v (and store them);
-                               // 0: they are current (left by the dense pass)
+    float2* partial;           // nblocks float-float sums of v (one per SM)
+    int32_t nblocks;
     float c;                   // c_push or c_fetch
     float eps_b;
     uint32_t round_key0[10];
@@ -29,18 +24,18 @@ struct MessageArgs {
     float* dst;
     int32_t* flag_out;         // may be null: 1 transmitted, 0 dropped
     float* vbar_out;           // may be null: the statistic vbar the decision used
+    uint32_t* decided;         // launch_message_decide: the decision
 };
 
-int32_t message_partial_blocks(int64_t P);
-
+// The decision and the copy (message_resolve_kernel), from a.partial.
 cudaError_t launch_message(const MessageArgs& a, int num_sms, cudaStream_t stream,
                            int64_t* launches);
-// The partials only (vbar_partial_kernel): for a decision the pass that
-// follows takes itself (message_decide).
-cudaError_t launch_message_partials(const MessageArgs& a, cudaStream_t stream, int64_t* launches);
+// a.partial from v.
+cudaError_t launch_message_sums(const MessageArgs& a, cudaStream_t stream, int64_t* launches);
+// The decision alone, into *a.decided, for the pass that follows.
+cudaError_t launch_message_decide(const MessageArgs& a, cudaStream_t stream, int64_t* launches);
 
-// The decision of one message from the nblocks partials vbar_partial_kernel
-// left, taken by one whole warp: lane l adds partials l, l + 32, ... in
+// The decision of one message from the nblocks partial sums of v, taken by one whole warp: lane l adds partials l, l + 32, ... in
 // order (eight loads in flight), then a fixed float-float shuffle tree,
 // vbar = fl32(sum / P) (ff_div_int), u = word 0 of Philox4x32-10 at counter
 // (2^32-1, client_word, n_lo, n_hi), the exact Eq. 9 test.  Every caller

@@ -167,12 +167,13 @@ struct fasgd_s {
                     cudaGetErrorString(st));
     }
     // Per-message B-FASGD: the gradient cache (lambda slots of cache_stride
-    // floats, allocated by the first message push) and the partial sums.
+    // floats, allocated by the first message push) and the sums of v.
     float* grad_cache = nullptr;
     int64_t cache_stride = 0;
-    float2* msg_partial = nullptr;
-    float2* msg_chunks = nullptr;   // chunk sums of v (128 parameters each)
-    bool msg_sums_valid = false;    // msg_chunks holds those of the current v
+    float2* msg_partial = nullptr;  // one sum of v per SM's share of the parameters,
+    float2* msg_fresh = nullptr;    //   a second set (formed before a pass that leaves its own),
+    uint32_t* msg_decided = nullptr;   // and the latest push's decision: one allocation
+    bool msg_sums_valid = false;    // msg_partial holds the sums of the current v
 
     // Per-tensor B-FASGD: the partition, its work items on the device, the
     // item sums of v and the decision of the latest call.
@@ -273,12 +274,13 @@ struct fasgd_s {
 
     cudaError_t ensure_message_scratch(bool cache) {
         cudaError_t st = cudaSuccess;
-        if (msg_partial == nullptr)
+        if (msg_partial == nullptr) {
             st = cudaMalloc(reinterpret_cast<void**>(&msg_partial),
-                            fasgd::kMessageMaxBlocks * sizeof(float2));
-        if (st == cudaSuccess && msg_chunks == nullptr) {
-            st = cudaMalloc(reinterpret_cast<void**>(&msg_chunks),
-                            (size_t)((P + fasgd::kVsumChunk - 1) / fasgd::kVsumChunk) * sizeof(float2));
+                            ((size_t)num_sms * 2 + 1) * sizeof(float2));
+            if (st == cudaSuccess) {
+                msg_fresh = msg_partial + num_sms;
+                msg_decided = reinterpret_cast<uint32_t*>(msg_fresh + num_sms);
+            }
             msg_sums_valid = false;
         }
         if (st == cudaSuccess && cache && grad_cache == nullptr) {
@@ -304,9 +306,7 @@ struct fasgd_s {
         a.v = v;
         a.P = P;
         a.partial = msg_partial;
-        a.nblocks = fasgd::message_partial_blocks(P);
-        a.chunks = msg_chunks;
-        a.from_v = msg_sums_valid ? 0 : 1;
+        a.nblocks = num_sms;
         a.c = c;
         a.eps_b = eps_b;
         fasgd::philox_key_schedule(seed, a.round_key0, a.round_key1);
@@ -327,9 +327,13 @@ struct fasgd_s {
                                float* vbar_out = nullptr) {
         const uint64_t n = counter != nullptr ? (*counter)[(size_t)client] : 0;
         const fasgd::MessageArgs a = message_args(stream_id, client, src, dst, flag, c, n, vbar_out);
-        cudaError_t st = fasgd::launch_message(a, num_sms, stream, &launches);
+        cudaError_t st = cudaSuccess;
+        if (!msg_sums_valid) st = fasgd::launch_message_sums(a, stream, &launches);
         if (st == cudaSuccess) {
             msg_sums_valid = true;
+            st = fasgd::launch_message(a, num_sms, stream, &launches);
+        }
+        if (st == cudaSuccess) {
             if (counter != nullptr) (*counter)[(size_t)client] = n + 1;
         }
         return st;
@@ -373,9 +377,9 @@ struct fasgd_s {
         cudaFree(dev_err);
         cudaFree(grad_cache);
         cudaFree(msg_partial);
-        cudaFree(msg_chunks);
-        msg_chunks = nullptr;
         msg_sums_valid = false;
+        msg_fresh = nullptr;
+        msg_decided = nullptr;
         grad_cache = nullptr;
         msg_partial = nullptr;
         free_tensors();
@@ -854,9 +858,8 @@ int fasgd_apply_pending(fasgd_t* h, int32_t K) {
         } else if (first.kind == kMessage) {
             // Decide against the mean of v now, refresh the client's cache
             // slot if the push is transmitted, then apply the slot.  Under the
-            // FASGD rules the pass itself takes the decision from the
-            // statistic's partials and, if transmitted, applies the pushed
-            // gradient while copying it into the slot.
+            // FASGD rules the pass, if the push is transmitted, applies the
+            // pushed gradient while copying it into the slot.
             float* slot = h->grad_cache + (size_t)first.client * (size_t)h->cache_stride;
             const uint64_t count0 = h->push_count[(size_t)first.client];
             fasgd::DenseArgs a;
@@ -873,13 +876,19 @@ int fasgd_apply_pending(fasgd_t* h, int32_t K) {
             a.K = 1;
             cudaError_t st;
             if (rule != fasgd::kRuleSgd) {
-                const fasgd::MessageArgs m =
+                fasgd::MessageArgs m =
                     h->message_args(0, first.client, first.grad, slot, first.flag, h->c_push,
                                     count0, nullptr);
-                st = fasgd::launch_message_partials(m, h->stream, &h->launches);
+                // The sums are current: decide from them.  Else form them; the
+                // pass then decides.
+                m.decided = h->msg_decided;
+                if (!h->msg_sums_valid) m.partial = h->msg_fresh;
+                st = h->msg_sums_valid ? fasgd::launch_message_decide(m, h->stream, &h->launches)
+                                       : fasgd::launch_message_sums(m, h->stream, &h->launches);
                 if (st == cudaSuccess) {
-                    a.vsum = h->msg_chunks;   // keep the chunk sums current
-                    a.msg.partial = m.partial;
+                    a.msg.decided = h->msg_sums_valid ? h->msg_decided : nullptr;
+                    a.msg.fresh = h->msg_fresh;
+                    a.msg.partial = h->msg_partial;
                     a.msg.nblocks = m.nblocks;
                     a.msg.c = m.c;
                     a.msg.eps_b = m.eps_b;

@@ -49,21 +49,41 @@ __device__ __forceinline__ void ff_warp_sum(float& h, float& l) {
     }
 }
 
-// The sum of one 128-parameter chunk of v, as a float-float pair, from this
-// lane's four consecutive values (lane l holds parameters 4l .. 4l + 3 of the
-// chunk; values past the end are passed as 0, which adds nothing): TwoSum in
-// the order x, y, z, w, renormalised, then the fixed warp tree.  Every lane
-// ends with the same pair; the bits depend only on the values.
-__device__ __forceinline__ float2 chunk_sum4(float4 v) {
-    float hi = 0.f, lo = 0.f;
-    two_sum_acc(hi, lo, v.x);
-    two_sum_acc(hi, lo, v.y);
-    two_sum_acc(hi, lo, v.z);
-    two_sum_acc(hi, lo, v.w);
-    float h, l;
-    two_sum(hi, lo, h, l);
-    ff_warp_sum(h, l);
-    return make_float2(h, l);
+// One thread's running float-float sum of quads of v: the four values by
+// TwoSum in the order x, y, z, w, then one pair addition; every 32 quads the
+// pair moves into a second one, so that no chain of additions grows long
+// (at 25M parameters a thread adds 81 quads: 32 + 3 steps; at 2^28, 32 + 27).
+// The same quads in the same order give the same bits wherever it runs.
+struct VSum {
+    float h = 0.f, l = 0.f, hh = 0.f, ll = 0.f;
+    uint32_t count = 0;
+    __device__ __forceinline__ void add(const float4& v) {
+        float s, e, t, lo;
+        two_sum(v.x, v.y, s, lo);
+        two_sum(s, v.z, t, e);
+        lo = __fadd_rn(lo, e);
+        two_sum(t, v.w, s, e);
+        lo = __fadd_rn(lo, e);
+        ff_add(h, l, s, lo);
+        if ((++count & 31u) == 0) {
+            ff_add(hh, ll, h, l);
+            h = l = 0.f;
+        }
+    }
+    // The warp's total, the same in every lane.
+    __device__ __forceinline__ float2 warp_total() {
+        ff_add(hh, ll, h, l);
+        ff_warp_sum(hh, ll);
+        return make_float2(hh, ll);
+    }
+};
+
+// The pairs of N warps added in order.
+template <int N>
+__device__ __forceinline__ float2 ordered_total(const float2* w) {
+    float2 t = make_float2(0.f, 0.f);
+    for (int i = 0; i < N; ++i) ff_add(t.x, t.y, w[i].x, w[i].y);
+    return t;
 }
 
 // fl32((h + l) / s) for a float-float pair (h >= 0, |l| <= ulp(h)) and an
