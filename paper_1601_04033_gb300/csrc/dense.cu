@@ -360,8 +360,15 @@ cudaError_t launch_ch(const DenseArgs& a, int stages, int num_sms, cudaStream_t 
 // default cache policy here.
 constexpr int kDirectThreads = 128;
 constexpr int kDirectTilesPerSm = 8;
+// Blocks of the grid at most, per SM: up to 1.25M parameters a thread has one
+// quad, beyond that the last round is short.  The kernel is built for K = 1, up
+// to 4 and up to 8 gradients at a time: 40 registers instead of 64 at K = 1, so
+// 12 blocks per SM are resident instead of 8.  Push + apply + pull at 1.29M, with
+// 8 blocks per SM and one kernel for all K -> now: K = 1 10.7 -> 8.3 us, K = 3
+// 13.8 -> 12.4, K = 8 18.8 -> 18.0, exact K = 1 12.3 -> 9.2.
+constexpr int kDirectBlocksPerSm = 16;
 
-template <int RULE, int ARITH>
+template <int RULE, int ARITH, int KMAX>
 __global__ void __launch_bounds__(kDirectThreads)
 fasgd_direct_kernel(const __grid_constant__ DenseArgs a) {
     constexpr bool FAS = RULE != kRuleSgd;
@@ -381,14 +388,14 @@ fasgd_direct_kernel(const __grid_constant__ DenseArgs a) {
                 v = *reinterpret_cast<const float4*>(a.v + e);
             }
             Guard<ARITH> guard;
-            for (int k0 = 0; k0 < a.K; k0 += 8) {
-                float4 g[8];
+            for (int k0 = 0; k0 < (KMAX == 1 ? 1 : a.K); k0 += KMAX) {
+                float4 g[KMAX];
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (k0 + j < a.K) g[j] = *reinterpret_cast<const float4*>(a.grad[k0 + j] + e);
+                for (int j = 0; j < KMAX; ++j)
+                    if (KMAX == 1 || k0 + j < a.K) g[j] = *reinterpret_cast<const float4*>(a.grad[k0 + j] + e);
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (k0 + j < a.K) update4<RULE, ARITH>(th, n, b, v, g[j], a.coef[k0 + j], a.sp, guard);
+                for (int j = 0; j < KMAX; ++j)
+                    if (KMAX == 1 || k0 + j < a.K) update4<RULE, ARITH>(th, n, b, v, g[j], a.coef[k0 + j], a.sp, guard);
             }
             if (!guard.ok()) redo_quad<RULE>(a, a.grad[0], e, th, n, b, v);
             *reinterpret_cast<float4*>(a.theta + e) = th;
@@ -426,8 +433,11 @@ template <int RULE, int ARITH>
 cudaError_t launch_direct(const DenseArgs& a, int num_sms, cudaStream_t stream) {
     const int64_t nq = (a.P + 3) / 4;
     int64_t grid = (nq + kDirectThreads - 1) / kDirectThreads;
-    if (grid > 8 * (int64_t)num_sms) grid = 8 * (int64_t)num_sms;
-    return launch_pdl(fasgd_direct_kernel<RULE, ARITH>, (unsigned)grid, kDirectThreads, 0, stream, a);
+    if (grid > kDirectBlocksPerSm * (int64_t)num_sms) grid = kDirectBlocksPerSm * (int64_t)num_sms;
+    const auto kernel = a.K == 1   ? fasgd_direct_kernel<RULE, ARITH, 1>
+                        : a.K <= 4 ? fasgd_direct_kernel<RULE, ARITH, 4>
+                                   : fasgd_direct_kernel<RULE, ARITH, 8>;
+    return launch_pdl(kernel, (unsigned)grid, kDirectThreads, 0, stream, a);
 }
 
 template <int RULE, int ARITH>
