@@ -6,10 +6,16 @@
 // Indices in one list are strictly ascending, so no two threads touch the
 // same parameter and no atomics are needed.  The count is read on the device
 // (it was produced there by the select kernels), so no host round trip sits
-// between select and apply.  A persistent grid walks the list; each warp
-// takes 32 consecutive entries per step, four steps per iteration, so the
-// index and value loads are coalesced and four gathers per array are in
-// flight per thread.
+// between select and apply.  A persistent grid walks the list; each warp takes
+// 32 kUnroll consecutive entries per iteration, so the index and value loads are
+// coalesced and kUnroll gathers per array are in flight per thread.
+//
+// Bound by HBM at the granularity of sectors: at 20 % kept almost every sector
+// of theta, n, b, v is read and most are written (25M: 725 MB in about 117 us, 6.2
+// TB/s), and by latency for small models: with the first list entries asked for
+// beside the count and two entries per thread instead of four, four exchanges
+// take 107 instead of 112 us at 1.29M, 154 instead of 177 at 3M, 271 instead of
+// 277 at 6M.
 
 #include <atomic>
 
@@ -21,45 +27,51 @@ namespace fasgd {
 namespace {
 
 constexpr int kSparseThreads = 256;
-constexpr int kUnroll = 4;
 
-template <int RULE, bool EXACT>
-__global__ void __launch_bounds__(kSparseThreads) fasgd_sparse_kernel(const __grid_constant__ SparseArgs a) {
+// AHEAD: the first step's list entries are loaded beside the count.
+template <int RULE, bool EXACT, int kUnroll, bool AHEAD>
+__global__ void __launch_bounds__(kSparseThreads, !AHEAD ? 1 : EXACT ? 6 : 8) fasgd_sparse_kernel(const __grid_constant__ SparseArgs a) {
     constexpr bool FAS = RULE != kRuleSgd;
-    pdl_wait();
-    pdl_trigger();
-    int64_t count = a.count_max;
-    if (a.count_dev != nullptr) {
-        const int64_t c = *a.count_dev;
-        count = c;
-        if (c < 0 || c > a.count_max) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.err, 1);
-            count = c < 0 ? 0 : a.count_max;
-        }
-    }
     const int lane = threadIdx.x & 31;
     const int64_t warp_id = ((int64_t)blockIdx.x * kSparseThreads + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * kSparseThreads) >> 5;
-    for (int64_t base = warp_id * (32 * kUnroll); base < count; base += nwarps * (32 * kUnroll)) {
-        int32_t p[kUnroll];
-        float g[kUnroll];
-        bool ok[kUnroll];
+    pdl_wait();
+    pdl_trigger();
+    int64_t count = a.count_max;
+    if (a.count_dev != nullptr) count = *a.count_dev;
+    int32_t p[kUnroll], prev[kUnroll];
+    float g[kUnroll];
+    // This lane's entries of the step at `from`, those below `end`.
+    const auto load = [&](int64_t from, int64_t end) {
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) {
-            const int64_t i = base + u * 32 + lane;
-            ok[u] = false;
-            p[u] = 0;
-            g[u] = 0.f;
-            if (i < count) {
+            const int64_t i = from + u * 32 + lane;
+            if (i < end) {
                 p[u] = a.idx[i];
                 g[u] = a.val[i];
-                const int32_t prev = (i > 0) ? a.idx[i - 1] : -1;
+                prev[u] = i > 0 ? a.idx[i - 1] : -1;
+            }
+        }
+    };
+    const int64_t first = warp_id * (32 * kUnroll);
+    if (AHEAD) load(first, a.count_max);
+    if (a.count_dev != nullptr && (count < 0 || count > a.count_max)) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.err, 1);
+        count = count < 0 ? 0 : a.count_max;
+    }
+    for (int64_t base = first; base < count; base += nwarps * (32 * kUnroll)) {
+        bool ok[kUnroll];
+        if (!AHEAD || base != first) load(base, count);
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+            ok[u] = base + u * 32 + lane < count;
+            if (ok[u]) {
                 if (p[u] < 0 || (int64_t)p[u] >= a.P) {
                     atomicOr(a.err, 2);
-                } else if (p[u] <= prev) {
+                    ok[u] = false;
+                } else if (p[u] <= prev[u]) {
                     atomicOr(a.err, 4);
-                } else {
-                    ok[u] = true;
+                    ok[u] = false;
                 }
             }
         }
@@ -93,14 +105,14 @@ __global__ void __launch_bounds__(kSparseThreads) fasgd_sparse_kernel(const __gr
     }
 }
 
-template <int RULE, bool EXACT>
-cudaError_t launch_rule(const SparseArgs& a, int num_sms, cudaStream_t stream) {
+template <int RULE, bool EXACT, int kUnroll, bool AHEAD>
+cudaError_t launch_form(const SparseArgs& a, int num_sms, cudaStream_t stream) {
     // Resident blocks per SM, looked up once (the grid is only capped by it).
     static std::atomic<int> cached{0};
     int blocks_per_sm = cached.load(std::memory_order_relaxed);
     if (blocks_per_sm == 0) {
         cudaError_t st = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &blocks_per_sm, fasgd_sparse_kernel<RULE, EXACT>, kSparseThreads, 0);
+            &blocks_per_sm, fasgd_sparse_kernel<RULE, EXACT, kUnroll, AHEAD>, kSparseThreads, 0);
         if (st != cudaSuccess) return st;
         if (blocks_per_sm < 1) blocks_per_sm = 1;
         cached.store(blocks_per_sm, std::memory_order_relaxed);
@@ -111,7 +123,19 @@ cudaError_t launch_rule(const SparseArgs& a, int num_sms, cudaStream_t stream) {
     const int64_t cap = (int64_t)num_sms * blocks_per_sm;
     if (want > cap) want = cap;
     if (want < 1) want = 1;
-    return launch_pdl(fasgd_sparse_kernel<RULE, EXACT>, (unsigned)want, kSparseThreads, 0, stream, a);
+    return launch_pdl(fasgd_sparse_kernel<RULE, EXACT, kUnroll, AHEAD>, (unsigned)want, kSparseThreads, 0, stream, a);
+}
+
+// Models up to 10M parameters: two entries per thread, the first step's ahead of
+// the count, as many warps as fit (latency shows there).  Larger ones: four after
+// it and registers to hold them, two blocks per SM: with fewer bytes in flight
+// HBM serves the scattered sectors faster (four exchanges at 25M: 957 us against
+// 980 with the small form and 975 with six blocks; 7M 319 against 313; 12M 499
+// against 502; 16M 640 against 650).
+template <int RULE, bool EXACT>
+cudaError_t launch_rule(const SparseArgs& a, int num_sms, cudaStream_t stream) {
+    return a.count_max <= 10'000'000 ? launch_form<RULE, EXACT, 2, true>(a, num_sms, stream)
+                                     : launch_form<RULE, EXACT, 4, false>(a, num_sms, stream);
 }
 
 constexpr int kScatterUnroll = 8;
@@ -163,8 +187,7 @@ __global__ void __launch_bounds__(kSparseThreads) fetch_scatter_kernel(const __g
 }  // namespace
 
 cudaError_t launch_scatter(const ScatterArgs& a, int num_sms, cudaStream_t stream) {
-    const int64_t per_block = (int64_t)kSparseThreads * kScatterUnroll;
-    int64_t want = (a.count_max + per_block - 1) / per_block;
+    int64_t want = (a.count_max + kSparseThreads - 1) / kSparseThreads;
     const int64_t cap = (int64_t)(num_sms > 0 ? num_sms : 1) * 8;
     if (want > cap) want = cap;
     if (want < 1) want = 1;
