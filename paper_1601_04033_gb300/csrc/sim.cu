@@ -8,12 +8,15 @@
 // exact, u = the top 23 bits of word (p mod 4) of Philox4x32-10 at counter
 // (p div 4, client + 2^30, n, n >> 32) -- every operation exact or rounded
 // once, so the result is reproducible bit for bit.
+// All three kernels are launched as programmatic dependents (pdl.cuh).
 // Loss: the terms h (theta - star)^2 in fp32, summed over a fixed partition
 // (per thread an fp32 sum plus its exact TwoSum errors, then fixed fp64
 // combines), times 1/2.
 
 #include "eq9.cuh"
 #include "kernels.cuh"
+#include "pdl.cuh"
+#include "twosum.cuh"
 
 namespace fasgd {
 namespace {
@@ -33,6 +36,8 @@ __device__ __forceinline__ float sim_grad_one(float theta, float h, float star, 
 }
 
 __global__ void __launch_bounds__(kSimThreads) sim_grad_kernel(const __grid_constant__ SimGradArgs a) {
+    pdl_wait();
+    pdl_trigger();
     const int64_t nq = (a.P + 3) >> 2;
     const int64_t stride = (int64_t)gridDim.x * kSimThreads;
     for (int64_t q = (int64_t)blockIdx.x * kSimThreads + threadIdx.x; q < nq; q += stride) {
@@ -59,16 +64,10 @@ __global__ void __launch_bounds__(kSimThreads) sim_grad_kernel(const __grid_cons
     }
 }
 
-__device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
-    const float t = __fadd_rn(hi, x);
-    const float xp = __fsub_rn(t, hi);
-    const float hp = __fsub_rn(t, xp);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, hp), __fsub_rn(x, xp)));
-    hi = t;
-}
-
 __global__ void __launch_bounds__(kSimThreads) sim_loss_partial_kernel(const __grid_constant__ SimLossArgs a) {
     __shared__ double smem[kSimThreads / 32];
+    pdl_wait();
+    pdl_trigger();
     const int64_t chunk = (a.P + kLossBlocks - 1) / kLossBlocks;
     const int64_t p0 = (int64_t)blockIdx.x * chunk;
     const int64_t p1 = p0 + chunk < a.P ? p0 + chunk : a.P;
@@ -91,8 +90,15 @@ __global__ void __launch_bounds__(kSimThreads) sim_loss_partial_kernel(const __g
 
 __global__ void sim_loss_final_kernel(const __grid_constant__ SimLossArgs a) {
     const int lane = threadIdx.x;
+    pdl_wait();
+    pdl_trigger();
+    // Every load before the additions, which keep their order.
+    double x[kLossBlocks / 32];
+#pragma unroll
+    for (int b = 0; b < kLossBlocks / 32; ++b) x[b] = a.partial[32 * b + lane];
     double s = 0.0;
-    for (int b = lane; b < kLossBlocks; b += 32) s += a.partial[b];
+#pragma unroll
+    for (int b = 0; b < kLossBlocks / 32; ++b) s += x[b];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(kFull, s, off);
     if (lane == 0) *a.loss = 0.5 * s;
@@ -105,16 +111,12 @@ cudaError_t launch_sim_grad(const SimGradArgs& a, int num_sms, cudaStream_t stre
     const int64_t cap = (int64_t)(num_sms > 0 ? num_sms : 1) * 8;
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
-    sim_grad_kernel<<<(unsigned)grid, kSimThreads, 0, stream>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(sim_grad_kernel, (unsigned)grid, kSimThreads, 0, stream, a);
 }
 
 cudaError_t launch_sim_loss(const SimLossArgs& a, cudaStream_t stream) {
-    sim_loss_partial_kernel<<<kLossBlocks, kSimThreads, 0, stream>>>(a);
-    cudaError_t st = cudaGetLastError();
-    if (st != cudaSuccess) return st;
-    sim_loss_final_kernel<<<1, 32, 0, stream>>>(a);
-    return cudaGetLastError();
+    const cudaError_t st = launch_pdl(sim_loss_partial_kernel, kLossBlocks, kSimThreads, 0, stream, a);
+    return st != cudaSuccess ? st : launch_pdl(sim_loss_final_kernel, 1, 32, 0, stream, a);
 }
 
 }  // namespace fasgd

@@ -59,6 +59,29 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long x)
     return (unsigned long long)p0 + ((unsigned long long)p1 << 21) + ((unsigned long long)p2 << 42);
 }
 
+__device__ __forceinline__ void acc4(float& hi, float& lo, const float4& x) {
+    two_sum_acc(hi, lo, x.x);
+    two_sum_acc(hi, lo, x.y);
+    two_sum_acc(hi, lo, x.z);
+    two_sum_acc(hi, lo, x.w);
+}
+
+// The threads' pairs through a fixed float-float tree; the result is valid in
+// thread 0.  Called by every thread of the block.
+__device__ __forceinline__ float2 block_total(float hi, float lo, float2* smem) {
+    const int tid = threadIdx.x;
+    float h, l;
+    two_sum(hi, lo, h, l);
+    ff_warp_sum(h, l);
+    if ((tid & 31) == 0) smem[tid >> 5] = make_float2(h, l);
+    __syncthreads();
+    float2 sum = make_float2(0.f, 0.f);
+    if (tid == 0)
+        for (int w = 0; w < kItemThreads / 32; ++w) ff_add(sum.x, sum.y, smem[w].x, smem[w].y);
+    __syncthreads();
+    return sum;
+}
+
 // The sum of v over one item as a float-float pair, the same bits wherever
 // it is formed (the partial kernel, or the apply kernel after it rewrote the
 // item): thread tid adds, in this order and with TwoSum, the head element
@@ -86,24 +109,10 @@ __device__ float2 item_v_sum(const TensorItem& it, const float* v, float2* smem)
                 if (q + k * kItemThreads < qe) x[k] = v4[q + k * kItemThreads];
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (q + k * kItemThreads < qe) {
-                    two_sum_acc(hi, lo, x[k].x);
-                    two_sum_acc(hi, lo, x[k].y);
-                    two_sum_acc(hi, lo, x[k].z);
-                    two_sum_acc(hi, lo, x[k].w);
-                }
+                if (q + k * kItemThreads < qe) acc4(hi, lo, x[k]);
         }
     }
-    float h, l;
-    two_sum(hi, lo, h, l);
-    ff_warp_sum(h, l);
-    if ((tid & 31) == 0) smem[tid >> 5] = make_float2(h, l);
-    __syncthreads();
-    float2 sum = make_float2(0.f, 0.f);
-    if (tid == 0)
-        for (int w = 0; w < kItemThreads / 32; ++w) ff_add(sum.x, sum.y, smem[w].x, smem[w].y);
-    __syncthreads();
-    return sum;
+    return block_total(hi, lo, smem);
 }
 
 __global__ void __launch_bounds__(kItemThreads) tensor_partial_kernel(const __grid_constant__ TensorArgs a) {
@@ -387,19 +396,22 @@ __global__ void __launch_bounds__(kTensorResolveThreads) budget_resolve_kernel(c
     }
 }
 
+// Returns the new v.
 template <int RULE, int ARITH>
-__device__ __forceinline__ void update1(const RangeArgs& a, int64_t p) {
-    float th = a.theta[p];
+__device__ __forceinline__ float update1(const RangeArgs& a, int64_t p) {
+    float th = a.theta[p], v = 0.f;
     if (RULE == kRuleSgd) {
         sgd_update(th, a.grad[p], a.coef);
     } else {
-        float n = a.n[p], b = a.b[p], v = a.v[p];
+        float n = a.n[p], b = a.b[p];
+        v = a.v[p];
         rule_update<ARITH, RULE == kRuleFasgdStd>(th, n, b, v, a.grad[p], a.coef, a.sp);
         a.n[p] = n;
         a.b[p] = b;
         a.v[p] = v;
     }
     a.theta[p] = th;
+    return v;
 }
 
 // A quad whose exact arithmetic left the range of its fast form.
@@ -439,11 +451,21 @@ __global__ void __launch_bounds__(kItemThreads) tensor_apply_kernel(const __grid
         if (!a.sent[it.tensor]) continue;
         const int64_t s = it.start, e = s + it.len;
         const int64_t qs = (s + 3) >> 2, qe = e >> 2;
+        float hi = 0.f, lo = 0.f;   // the new v, added in item_v_sum's order
         if (4 * qs >= e) {
-            for (int64_t p = s + tid; p < e; p += kItemThreads) update1<RULE, ARITH>(a, p);
+            for (int64_t p = s + tid; p < e; p += kItemThreads) {
+                const float v = update1<RULE, ARITH>(a, p);
+                if (FAS) two_sum_acc(hi, lo, v);
+            }
         } else {
-            if (tid < 4 * qs - s) update1<RULE, ARITH>(a, s + tid);
-            if (tid < e - 4 * qe) update1<RULE, ARITH>(a, 4 * qe + tid);
+            if (tid < 4 * qs - s) {
+                const float v = update1<RULE, ARITH>(a, s + tid);
+                if (FAS) two_sum_acc(hi, lo, v);
+            }
+            if (tid < e - 4 * qe) {
+                const float v = update1<RULE, ARITH>(a, 4 * qe + tid);
+                if (FAS) two_sum_acc(hi, lo, v);
+            }
             for (int64_t q0 = qs + tid; q0 < qe; q0 += 2 * kItemThreads) {
                 const int64_t q1 = q0 + kItemThreads;
                 const bool two = q1 < qe;
@@ -472,6 +494,7 @@ __global__ void __launch_bounds__(kItemThreads) tensor_apply_kernel(const __grid
                     st4(a.n, q0, n0);
                     st4(a.b, q0, b0);
                     st4(a.v, q0, v0);
+                    acc4(hi, lo, v0);
                 }
                 if (two) {
                     Guard<ARITH> guard1;
@@ -482,13 +505,13 @@ __global__ void __launch_bounds__(kItemThreads) tensor_apply_kernel(const __grid
                         st4(a.n, q1, n1);
                         st4(a.b, q1, b1);
                         st4(a.v, q1, v1);
+                        acc4(hi, lo, v1);
                     }
                 }
             }
         }
         if (FAS && a.partial != nullptr) {
-            __syncthreads();    // the block's writes of v are visible to the block
-            const float2 sum = item_v_sum(it, a.v, smem);
+            const float2 sum = block_total(hi, lo, smem);
             if (tid == 0) a.partial[i] = sum;
         }
     }
