@@ -5,7 +5,7 @@
 // Philox counter streams (bit 31 of the client word).
 //
 // Two kernels, on the caller's stream:
-//   1. decide:  per tile of 4096 parameters (one block, 1024 per warp), draw u_p
+//   1. decide:  per tile of 4096 parameters (one block), draw u_p
 //               (Philox4x32-10), take the Eq. 9 decision against v_p, store one
 //               bit per parameter and the tile's count of kept entries;
 //   2. compact: per tile, the sum of the earlier tiles' counts gives its place
@@ -31,14 +31,15 @@
 // Blocks of 128 threads, eight per SM: a tile is small beside the SM's share
 // at 1.3M parameters already, and the last wave is short.
 // The whole select of 25M parameters at 20 % kept: 57 -> about 46 us with the
-// scan kernel gone (exchange of four clients 1068 -> 976 us); of 1.29M: four
-// exchanges 135 -> 110 us, from Python.
+// scan kernel gone (exchange of four clients 1068 -> 976 us).
 //
 // Tried as one kernel (the compaction's memory time under the decision's ALU
 // time): warps that wait for the counts of earlier tiles took 140 us per 25M
 // one tile each (the polls of the same few words), and 57 us persistent with
 // three decided tiles in hand (tickets for the tiles, one address, cost 2.3 ns
 // an atomic).  Values prefetched into L2 by decide: 1014 against 986 us.
+
+#include <type_traits>
 
 #include "eq9.cuh"
 #include "kernels.cuh"
@@ -48,25 +49,27 @@
 namespace fasgd {
 namespace {
 
-// Both kernels: a span of 1024 parameters per warp.
+// A span of 1024 parameters is one word of bits per lane of a warp.  compact: a
+// span per warp.  decide: QUADS quads per lane, so that a warp takes a span (8),
+// a half or a quarter of one.
 constexpr int kSpan = 1024;
 constexpr int kThreads = kSelectTile / 32;
 constexpr int kWarps = kThreads / 32;
-constexpr int kQuads = kSpan / 128;               // quads per lane of the decision
 constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ uint32_t smem_address(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// This lane's quads of v in the warp's span at `start` (zero past P).
-__device__ __forceinline__ void load_quads(float4 (&q)[kQuads], const float* v, int64_t start, int64_t P,
+// This lane's quads of v in the warp's parameters from `start` (zero past P).
+template <int QUADS>
+__device__ __forceinline__ void load_quads(float4 (&q)[QUADS], const float* v, int64_t start, int64_t P,
                                           int lane) {
     const int64_t e = start + 4 * lane;
-    if (start + kSpan <= P) {
+    if (start + 128 * QUADS <= P) {
 #pragma unroll
-        for (int it = 0; it < kQuads; ++it) q[it] = __ldcs(reinterpret_cast<const float4*>(v + e + 128 * it));
+        for (int it = 0; it < QUADS; ++it) q[it] = __ldcs(reinterpret_cast<const float4*>(v + e + 128 * it));
     } else {
 #pragma unroll
-        for (int it = 0; it < kQuads; ++it) {
+        for (int it = 0; it < QUADS; ++it) {
             const int64_t p = e + 128 * it;
             q[it].x = p < P ? v[p] : 0.f;
             q[it].y = p + 1 < P ? v[p + 1] : 0.f;
@@ -93,13 +96,13 @@ __device__ __forceinline__ void send_difference(uint32_t w0, uint32_t w1, float 
 }
 
 // Bit 4 it + j: parameter start + 128 it + 4 lane + j is sent.
-template <bool SCALE_D>
-__device__ __forceinline__ uint32_t quad_bits(const SelectArgs& a, const float4 (&v)[kQuads], uint32_t start,
+template <bool SCALE_D, int QUADS>
+__device__ __forceinline__ uint32_t quad_bits(const SelectArgs& a, const float4 (&v)[QUADS], uint32_t start,
                                               int lane) {
     const Pair c = pair(a.c, a.c), eps_b = pair(a.eps_b, a.eps_b);
     uint32_t bits = 0;
 #pragma unroll
-    for (int it = kQuads - 1; it >= 0; --it) {
+    for (int it = QUADS - 1; it >= 0; --it) {
         const uint32_t e = start + 128 * it + 4 * lane;   // P < 2^31
         const Philox4 r = philox4x32_10(e >> 2, a.client_word, a.push_lo, a.push_hi, a.round_key0, a.round_key1);
         float s[4];
@@ -131,34 +134,44 @@ __device__ __forceinline__ uint32_t lane_word(uint32_t x, int lane) {
 }
 
 // SCALE_D: the form of the Eq. 9 test for this call's c (send_form).
-template <bool SCALE_D>
-__global__ void __launch_bounds__(kThreads, 8) bfasgd_decide_kernel(const __grid_constant__ SelectArgs a) {
-    __shared__ int32_t warp_cnt[kWarps];
+template <bool SCALE_D, int QUADS>
+__global__ void __launch_bounds__(kSelectTile / (4 * QUADS), QUADS) bfasgd_decide_kernel(const __grid_constant__ SelectArgs a) {
+    constexpr int kDecideWarps = kSelectTile / (128 * QUADS), kParts = 8 / QUADS;   // warps per span
+    __shared__ int32_t warp_cnt[kDecideWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t start = (int64_t)blockIdx.x * kSelectTile + warp * kSpan;
+    const int64_t start = (int64_t)blockIdx.x * kSelectTile + warp * (128 * QUADS);
     pdl_wait();
     pdl_trigger();
-    float4 v[kQuads];
+    float4 v[QUADS];
     load_quads(v, a.v, start, a.P, lane);
     uint32_t bits = quad_bits<SCALE_D>(a, v, (uint32_t)start, lane);
-    if (start + kSpan > a.P) {   // parameters past P are never sent
+    if (start + 128 * QUADS > a.P) {   // parameters past P are never sent
 #pragma unroll
-        for (int it = 0; it < kQuads; ++it) {
+        for (int it = 0; it < QUADS; ++it) {
             const int64_t left = a.P - (start + 128 * it + 4 * lane);
             const uint32_t keep = left >= 4 ? 0xfu : left <= 0 ? 0u : (1u << left) - 1u;
             bits &= ~((~keep & 0xfu) << (4 * it));
         }
     }
-    a.mask[(start >> 5) + lane] = bits;
+    // This warp's part of the lane's word of the span (quads 32 it + lane).
+    using Part = typename std::conditional<QUADS == 8, uint32_t,
+                                           typename std::conditional<QUADS == 4, uint16_t, uint8_t>::type>::type;
+    reinterpret_cast<Part*>(a.mask)[kParts * ((start >> 10) * 32 + lane) + warp % kParts] = (Part)bits;
     const int n = (int)__reduce_add_sync(kFull, (uint32_t)__popc(bits));
     if (lane == 0) warp_cnt[warp] = n;
     __syncthreads();
     if (threadIdx.x == 0) {
         int32_t t = 0;
 #pragma unroll
-        for (int w = 0; w < kWarps; ++w) t += warp_cnt[w];
+        for (int w = 0; w < kDecideWarps; ++w) t += warp_cnt[w];
         a.tile_count[blockIdx.x] = (uint16_t)t;
     }
+}
+
+template <int QUADS>
+cudaError_t launch_decide(const SelectArgs& a, cudaStream_t stream) {
+    const auto kernel = send_form(a.c) ? bfasgd_decide_kernel<true, QUADS> : bfasgd_decide_kernel<false, QUADS>;
+    return launch_pdl(kernel, (unsigned)a.ntiles, kSelectTile / (4 * QUADS), 0, stream, a);
 }
 
 constexpr int kScanThreads = 1024;
@@ -287,12 +300,13 @@ __global__ void __launch_bounds__(kThreads, 8) bfasgd_compact_kernel(const __gri
         }
     }
     __syncthreads();
-    int64_t out = tile_out;
+    int32_t ahead = 0;
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) {
-        if (!SCANNED) out += warp_sum[w];
-        if (w < warp) out += warp_cnt[w];
+        if (!SCANNED) ahead += warp_sum[w];
+        if (w < warp) ahead += warp_cnt[w];
     }
+    const int64_t out = tile_out + ahead;
     int32_t* idx_out = a.idx + out;
     float* val_out = a.val + out;
 #pragma unroll
@@ -318,8 +332,15 @@ void select_key_schedule(SelectArgs& a, uint64_t seed) {
 }
 
 cudaError_t launch_select(const SelectArgs& a, cudaStream_t stream, int64_t* launches) {
-    const auto decide = send_form(a.c) ? bfasgd_decide_kernel<true> : bfasgd_decide_kernel<false>;
-    cudaError_t st = launch_pdl(decide, (unsigned)a.ntiles, kThreads, 0, stream, a);
+    // Quads per lane: with about two to seven tiles per SM shorter chains of
+    // draws per warp (and more warps) pay; below that a tile's 16 warps would
+    // crowd one SM while others idle, above it the SMs are full anyway.  Four
+    // exchanges with 2 / 4 / 8, us: 600,000 78 / 72 / 72, 800,000 83 / 84 / 80,
+    // 1.0M 88 / 92 / 93, 1.29M 90 / 101 / 107, 1.6M 109 / 109 / 119, 2M 122 /
+    // 117 / 127, 4M 207 / 196 / 196, 8M 372 / 356 / 350.
+    cudaError_t st = a.P > 850'000 && a.P <= 1'500'000     ? launch_decide<2>(a, stream)
+                     : a.P > 1'500'000 && a.P <= 4'500'000 ? launch_decide<4>(a, stream)
+                                                           : launch_decide<8>(a, stream);
     if (st != cudaSuccess) return st;
     ++*launches;
     const bool scan = a.ntiles > kScanTiles;

@@ -1,4 +1,5 @@
-"""The select kernels where their forms meet: around 8192 tiles of 4096
+"""The select kernels where their forms meet: around 850,000, 1.5M and 4.5M parameters
+(more parameters per warp of the decision), around 8192 tiles of 4096
 parameters (beyond, a scan kernel forms the tiles' places) and at densities on
 both sides of 256 kept entries per warp (fetched before or after the place is
 known), every list bit for bit against the oracle."""
@@ -15,6 +16,7 @@ SWITCH = 8192 * 4096
 
 
 @pytest.mark.parametrize("P,c", [(SWITCH, 40.0), (SWITCH + 1, 40.0), (SWITCH - 4095, 40.0)]
+                         + [(P, 40.0) for P in (850_000, 850_001, 1_500_000, 1_500_001, 4_500_000, 4_500_001)]
                          + [(P, c) for P in (1, 31, 1023, 1025, 4095, 4097, 40_961)
                             for c in (0.0, 1.0, 30.0, 90.0, 1e4, float(2.0 ** 80), float("inf"))])
 def test_select_lists_against_oracle(P, c):
