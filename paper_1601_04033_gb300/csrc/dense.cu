@@ -54,8 +54,8 @@ namespace {
 // Ring geometry per consumer count CONS (threads that compute; 512 or 256):
 // tiles of 4 CONS parameters, CONS + 32 threads per block (one producer
 // warp), 512 / CONS blocks per SM sharing 220 KB of shared memory.  A stage
-// holds the state's slices and min(K, CH) gradients' (not CH: K = 5 keeps three
-// tiles in flight where stages for eight gradients kept two).
+// holds the state's slices and min(K, CH) gradients'; how many stages a pass
+// uses is chosen with CH (launch_rule).
 template <int CONS> struct Geom {
     static constexpr int kTile = 4 * CONS;
     static constexpr int kThreads = CONS + 32;

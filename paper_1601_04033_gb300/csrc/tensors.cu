@@ -16,9 +16,9 @@
 // Then tensor_apply (a push: Eq. 4-8, or Eq. 1-2, on the transmitted
 // tensors) or tensor_copy (a fetch: theta into the client's copy) walks the
 // items of the transmitted tensors; the others cost one flag read.  The
-// apply re-forms the sums of the items it rewrote, in the partial kernel's
-// element order, so the item sums stay those of the current v and the next
-// decision skips the partial kernel (the host tracks when another pass has
+// apply adds the new v of the items it rewrites as it stores them, in the
+// partial kernel's element order, so the item sums stay those of the current v
+// and the next decision skips the partial kernel (the host tracks when another pass has
 // changed v and the sums must be formed afresh).  All four are launched as
 // programmatic dependents (pdl.cuh), so each one's launch overlaps the tail
 // of the kernel before it.
@@ -83,14 +83,12 @@ __device__ __forceinline__ float2 block_total(float hi, float lo, float2* smem) 
 }
 
 // The sum of v over one item as a float-float pair, the same bits wherever
-// it is formed (the partial kernel, or the apply kernel after it rewrote the
-// item): thread tid adds, in this order and with TwoSum, the head element
+// it is formed (here, or by the apply kernel as it rewrites the item): thread tid adds, in this order and with TwoSum, the head element
 // s + tid (before the first whole 16-byte quad), the tail element 4 qe + tid
 // (after the last), then quads qs + tid, qs + tid + 256, ...; the threads'
-// pairs go through a fixed float-float tree.  Four quads are loaded before
-// they are added, so a thread keeps four loads in flight.  Called by every
-// thread of the block; the result is valid in thread 0.  Plain loads (no
-// read-only path): the apply kernel reads values it has just written.
+// pairs go through a fixed float-float tree (block_total).  Four quads are
+// loaded before they are added, so a thread keeps four loads in flight.  Called
+// by every thread of the block; the result is valid in thread 0.
 __device__ float2 item_v_sum(const TensorItem& it, const float* v, float2* smem) {
     const int tid = threadIdx.x;
     const int64_t s = it.start, e = s + it.len;
@@ -436,9 +434,11 @@ __device__ __forceinline__ void st4(float* base, int64_t q, const float4& x) {
 // Eq. 4-8 (or Eq. 1-2) on every parameter of the transmitted tensors.  The
 // head and tail of an item (outside whole 16-byte quads) go element by
 // element; the quads two per thread per step, loads before stores.  When
-// partial is set (rules that change v), the block then re-forms the item's
-// sum of v from the values it just wrote (from L2), with the same element
-// order as the partial kernel, so the next decision needs no pass over v.
+// partial is set (rules that change v), each thread also adds its new v in
+// registers, in the partial kernel's element order, so the next decision needs
+// no pass over v.  Bound by HBM: 36 bytes per transmitted parameter (5.2M of
+// 25M: 186 MB in about 31 us; re-reading v from L2 for the sums, behind a block
+// barrier, took 33; four exchanges at 25M 250 -> 242 us, at 3M 111 -> 106).
 template <int RULE, int ARITH>
 __global__ void __launch_bounds__(kItemThreads) tensor_apply_kernel(const __grid_constant__ RangeArgs a) {
     constexpr bool FAS = RULE != kRuleSgd;
