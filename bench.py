@@ -654,9 +654,9 @@ def run_message(args, w, world, rank, local):
     peak, peak_kind = peaks()
     # A push: the cache refresh when sent (8 B per parameter) and the dense
     # K = 1 pass over the cache slot (36 B per parameter); the statistic
-    # comes from chunk sums the previous pass left (8 B read + 8 B written
-    # per 128 parameters), not from a pass over v.
-    push_bytes = P * (8 * s_frac + 36) + 16 * ((P + 127) // 128)
+    # comes from the sums the previous pass left (a pair per block), not from
+    # a pass over v.
+    push_bytes = P * (8 * s_frac + 36)
     achieved = push_bytes / (push_ms / 1e3) / 1e9
     return {
         "value": P * world / step_s, "ms_per_step": total_ms / args.steps,

@@ -16,9 +16,9 @@
 // parameters (128-bit shared loads), frees the stage as soon as its inputs
 // are in registers, applies the pushes, and stores the state with 128-bit
 // global stores.  A larger K runs as several stages per tile (the state travels
-// with the first one only).  Every block has the same number of whole tiles and
-// an equal piece of the rest (BlockShare); the last P mod 4 parameters go
-// through plain loads.  Passes of fewer than 8 tiles per SM use a plain grid
+// with the first one only).  Every block has an equal piece of what the whole
+// tiles leave over and the same number of tiles (BlockShare); the last P mod 4
+// parameters go through plain loads.  Passes of fewer than 8 tiles per SM use a plain grid
 // instead (one quad of parameters per thread, fasgd_direct_kernel).
 //
 // With SUMS (one push, a.msg.partial set) the pass applies a per-message push
@@ -303,9 +303,8 @@ fasgd_dense_kernel(const __grid_constant__ DenseArgs a, const Ring ring) {
         if (SUMS) vsum.add(v);
         return true;
     };
-    bool ok = true;
-    for (int64_t t = 0; t < share.whole && ok; ++t) ok = tile(std::true_type{}, share.offset(t), kTile);
-    if (ok && share.piece > 0) ok = tile(std::false_type{}, share.piece_start, share.piece);
+    bool ok = share.piece == 0 || tile(std::false_type{}, share.piece_start, share.piece);
+    for (int64_t t = 0; t < share.whole && ok; ++t) ok = tile(std::true_type{}, share.first + t * share.step, kTile);
     if (ok && blockIdx.x == gridDim.x - 1) {
         const float v = apply_ragged<RULE, ARITH>(a, tid, g0, copy_to);
         if (SUMS && tid < (int)(a.P & 3)) vsum.add(make_float4(v, 0.f, 0.f, 0.f));
