@@ -126,8 +126,8 @@ FASGD_API int fasgd_set_hparams(fasgd_t* h, float gamma, float beta, float eps, 
  * the first steps are large).  Measured: theta through 3.2 ending at 5.6e-3
  * is 7e-7 off (1.14 times the bound).  Use mode 1 there, and wherever runs
  * must reproduce exactly (closed-loop simulations, where feedback can
- * amplify ulp-level differences).  Mode 1 costs about 1.15x per dense pass
- * at K = 8 and 1.4x at K = 16 (25M parameters).  Errors: EINVAL, EAGAIN (pushes pending).
+ * amplify ulp-level differences).  Mode 1 costs about 1.1x per dense pass
+ * at K = 8 and 1.35x at K = 16 (25M parameters).  Errors: EINVAL, EAGAIN (pushes pending).
  */
 FASGD_API int fasgd_set_exact(fasgd_t* h, int32_t exact);
 

@@ -466,7 +466,7 @@ cudaError_t launch_rule(const DenseArgs& a, int num_sms, cudaStream_t stream) {
     //          4: 215 -> 206         5: 231 -> 217     6: 244 -> 229
     //          8: 253 -> 254         12: 316 -> 312    16: 375 (same)   32: 631 -> 601
     //   exact  3: 204 -> 190         4: 223 -> 207     5: 222 (same)
-    //          6: 238 -> 232         8: 281 (same)     16: 510 (same)
+    //          6: 238 -> 232         7: 260 -> 247     8: 273     16: 494
     //   SGD    K = 3: 103 -> 102     6: 148 -> 146     8: 182 -> 174
     //          12: 242 -> 232        16: 300 -> 287    32: 531 -> 512
     if constexpr (RULE == kRuleSgd) {
