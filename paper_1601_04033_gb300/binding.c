@@ -134,34 +134,39 @@ static const char* const names[F_COUNT] = {
     "fasgd_sim_quadratic_grad", "fasgd_sim_quadratic_loss"};
 
 /* install(namespace): keeps the ctypes functions of these names for the calls
- * this module does not take, and returns the names. */
+ * this module does not take, and returns the names.  A namespace that holds one
+ * of this module's own functions is refused whole: it would hand the call to
+ * itself without end. */
 static PyObject* py_install(PyObject* self, PyObject* space) {
-    PyObject* out;
-    (void)self;
+    PyObject *out, *f[F_COUNT];
     if (!PyDict_Check(space)) {
         PyErr_SetString(PyExc_TypeError, "install: a dict is expected");
         return NULL;
     }
-    out = PyList_New(0);
-    if (out == NULL) return NULL;
     for (int i = 0; i < F_COUNT; ++i) {
-        PyObject *f = PyDict_GetItemString(space, names[i]), *s, *old;
-        if (f == NULL) {
-            Py_DECREF(out);
+        f[i] = PyDict_GetItemString(space, names[i]);
+        if (f[i] == NULL) {
             PyErr_Format(PyExc_KeyError, "install: no %s", names[i]);
             return NULL;
         }
-        Py_INCREF(f);
-        old = slow[i];
-        slow[i] = f;
-        Py_XDECREF(old);
-        s = PyUnicode_FromString(names[i]);
+        if (PyCFunction_Check(f[i]) && PyCFunction_GET_SELF(f[i]) == self) {
+            PyErr_Format(PyExc_ValueError, "install: %s is this module's own", names[i]);
+            return NULL;
+        }
+    }
+    out = PyList_New(0);
+    if (out == NULL) return NULL;
+    for (int i = 0; i < F_COUNT; ++i) {
+        PyObject *s = PyUnicode_FromString(names[i]), *old = slow[i];
         if (s == NULL || PyList_Append(out, s) < 0) {
             Py_XDECREF(s);
             Py_DECREF(out);
             return NULL;
         }
         Py_DECREF(s);
+        Py_INCREF(f[i]);
+        slow[i] = f[i];
+        Py_XDECREF(old);
     }
     return out;
 }

@@ -263,8 +263,9 @@ try:
 except ImportError:
     _binding = None
 if _binding is not None:
-    for _name in _binding.install(globals()):
-        globals()[_name] = getattr(_binding, _name)
+    # The functions the module hands a call to when it does not take it itself.
+    _CTYPES = {_name: globals()[_name] for _name in _binding.install(globals())}
+    globals().update({_name: getattr(_binding, _name) for _name in _CTYPES})
 
 
 # ---------------------------------------------------------------------------

@@ -3,6 +3,7 @@ same results and refusals for every form of argument, on calls that the library
 rejects on the host (no GPU needed)."""
 
 import ctypes
+import inspect
 
 import numpy as np
 import pytest
@@ -14,51 +15,60 @@ except ImportError:                      # pragma: no cover - the library is not
 if f._binding is None:
     pytest.skip("built without Python's headers", allow_module_level=True)
 
-NAMES = f._binding.install({n: getattr(f, n) for n in f._binding.install(dict(vars(f)))})
+NAMES = sorted(f._CTYPES)
 COUNTS = {n: len(f.SIGNATURES[n][1]) - (n == "fasgd_pull") for n in NAMES}
 
 
-def through_ctypes(name, args):
-    if name == "fasgd_pull":
-        T = ctypes.c_int64()
-        return f.LIB.fasgd_pull(*args, ctypes.byref(T)), T.value
-    return getattr(f.LIB, name)(*args)
-
-
-def outcome(call, *args):
+def outcome(call, *args, **kwargs):
     try:
-        return call(*args)
+        return call(*args, **kwargs)
     except (TypeError, ctypes.ArgumentError):
         return "refused"
-
-
-@pytest.fixture(autouse=True)
-def slow_functions():
-    """The module's own fallbacks, restored after a test replaced them."""
-    f._binding.install({n: (lambda *a, _n=n: through_ctypes(_n, a)) for n in NAMES})
-    yield
-    f._binding.install({n: (lambda *a, _n=n: through_ctypes(_n, a)) for n in NAMES})
 
 
 @pytest.mark.parametrize("name", NAMES)
 def test_arguments_as_ctypes_takes_them(name):
     n = COUNTS[name]
-    fast = getattr(f._binding, name)
+    fast, slow = getattr(f, name), f._CTYPES[name]
+    assert fast is getattr(f._binding, name) and fast is not slow
     null = [None] + [0] * (n - 1)        # a null handle, or P = None / 0: rejected on the host
     for base in ([0] * n, null, [None] * n, [0] * (n - 1), [0] * (n + 1), []):
-        assert outcome(fast, *base) == outcome(through_ctypes, name, list(base)), base
+        assert outcome(fast, *base) == outcome(slow, *base), base
     for k in range(n):
         for bad in (None, 1.5, "x", True, -1, 1 << 70, np.int64(3), ctypes.c_void_p(), b"abc"):
             if k == 0 and bad is not None and bad != 1.5:
                 continue                 # would be taken for a handle or a size
             args = [0] * n
             args[k] = bad
-            assert outcome(fast, *args) == outcome(through_ctypes, name, args), (k, bad)
+            assert outcome(fast, *args) == outcome(slow, *args), (k, bad)
 
 
-def test_keywords_reach_the_python_function():
-    assert f.fasgd_apply_pending is f._binding.fasgd_apply_pending
+@pytest.mark.parametrize("name", NAMES)
+def test_keywords_and_odd_types_reach_the_functions_that_ship(name):
+    """Through the fallbacks fasgd.py installed, not stand-ins."""
+    params = list(inspect.signature(f._CTYPES[name]).parameters)
+    null = dict.fromkeys(params, 0)
+    assert outcome(getattr(f, name), **null) == f._CTYPES[name](**null)
+    assert outcome(getattr(f, name), **null, nonsense=1) == "refused"
+    assert outcome(getattr(f, name), None, *[ctypes.c_int64(0)] * (len(params) - 1)) == \
+        outcome(f._CTYPES[name], None, *[ctypes.c_int64(0)] * (len(params) - 1))
+
+
+def test_fallbacks_are_kept_whole():
+    """The module takes no function of its own as a fallback (a call would go
+    round without end), and a refused install changes nothing."""
+    own = {n: getattr(f._binding, n) for n in NAMES}
+    for space in (own, {**f._CTYPES, NAMES[-1]: own[NAMES[-1]]}, dict(vars(f))):
+        with pytest.raises(ValueError):
+            f._binding.install(space)
+    with pytest.raises(KeyError):
+        f._binding.install({})
+    assert f.fasgd_apply_pending(None, K=3) == f.EINVAL
     seen = []
-    f._binding.install({n: (lambda *a, _n=n, **k: seen.append((_n, a, k)) or 7) for n in NAMES})
-    assert f.fasgd_apply_pending(None, K=3) == 7
+    try:
+        f._binding.install({n: (lambda *a, _n=n, **k: seen.append((_n, a, k)) or 7) for n in NAMES})
+        assert f.fasgd_apply_pending(None, K=3) == 7
+    finally:
+        f._binding.install(f._CTYPES)
     assert seen == [("fasgd_apply_pending", (None,), {"K": 3})]
+    assert f.fasgd_apply_pending(None, K=3) == f.EINVAL
