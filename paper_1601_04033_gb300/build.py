@@ -88,13 +88,18 @@ def build(force: bool = False, verbose: bool = False, extra_flags: list | None =
 
 
 BINDING_SRC = os.path.join(PKG, "binding.c")
-BINDING = os.path.join(PKG, "_binding.so")
+# The name carries the interpreter's ABI and machine, so that every Python loads
+# only a module that was built for it.
+BINDING = os.path.join(PKG, "_binding" + sysconfig.get_config_var("EXT_SUFFIX"))
+_UNTAGGED = os.path.join(PKG, "_binding.so")   # what earlier versions built: any Python would load it
 
 
 def build_binding(force: bool = False) -> str | None:
     """Build the CPython module of the binding's hot calls (binding.c) against
     libfasgd.so; returns its path, or None where Python's headers are not
     installed (the binding then makes every call through ctypes)."""
+    if BINDING != _UNTAGGED and os.path.exists(_UNTAGGED):
+        os.remove(_UNTAGGED)
     include = sysconfig.get_paths()["include"]
     if not os.path.exists(os.path.join(include, "Python.h")):
         return None

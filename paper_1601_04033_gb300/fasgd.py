@@ -13,7 +13,9 @@ tensors (CUDA tensors for device arguments) and the current torch stream.
 from __future__ import annotations
 
 import ctypes
+import importlib
 import os
+import warnings
 
 from . import build as _build
 
@@ -257,11 +259,14 @@ def fasgd_last_error(h) -> str:
 
 # The hot entry points again, without ctypes' cost per call (binding.c): the
 # same names, arguments and results.  Absent where Python's headers were not
-# installed when the library was built; the functions above then serve.
+# installed when the library was built; the functions above then serve, as they
+# do, with a warning, where the module is there but does not load.
 try:
-    from . import _binding
-except ImportError:
+    _binding = importlib.import_module("._binding", __package__)
+except ImportError as _error:
     _binding = None
+    if not isinstance(_error, ModuleNotFoundError):
+        warnings.warn(f"{_error}: every call goes through ctypes", RuntimeWarning)
 if _binding is not None:
     # The functions the module hands a call to when it does not take it itself.
     _CTYPES = {_name: globals()[_name] for _name in _binding.install(globals())}

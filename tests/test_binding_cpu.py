@@ -3,7 +3,13 @@ same results and refusals for every form of argument, on calls that the library
 rejects on the host (no GPU needed)."""
 
 import ctypes
+import glob
 import inspect
+import os
+import shutil
+import subprocess
+import sys
+import sysconfig
 
 import numpy as np
 import pytest
@@ -72,3 +78,28 @@ def test_fallbacks_are_kept_whole():
         f._binding.install(f._CTYPES)
     assert seen == [("fasgd_apply_pending", (None,), {"K": 3})]
     assert f.fasgd_apply_pending(None, K=3) == f.EINVAL
+
+
+@pytest.mark.parametrize("name, warns", [("_binding.cpython-39-x86_64-linux-gnu.so", False),
+                                         ("_binding.so", True), ("_binding" + sysconfig.get_config_var("EXT_SUFFIX"), True)])
+def test_only_this_interpreters_module_is_loaded(tmp_path, name, warns):
+    """A module built for another Python is not looked at, and one that does not
+    load is reported; the calls go through ctypes either way."""
+    pkg = tmp_path / "paper_1601_04033_gb300"
+    pkg.mkdir()
+    for p in glob.glob(os.path.join(f._build.PKG, "*.py")):
+        shutil.copy(p, pkg)
+    os.symlink(f._build.LIB, pkg / "libfasgd.so")
+    (pkg / name).write_bytes(b"not a module")
+    code = ("import warnings\nwith warnings.catch_warnings(record=True) as w:\n"
+            "    warnings.simplefilter('always')\n    from paper_1601_04033_gb300 import fasgd as f\n"
+            "assert f._binding is None and f.fasgd_apply_pending(None, K=3) == f.EINVAL\n"
+            "print(sum('ctypes' in str(x.message) for x in w))")
+    r = subprocess.run([sys.executable, "-c", code], cwd=tmp_path, capture_output=True, text=True)
+    assert r.returncode == 0 and int(r.stdout) == warns, r.stdout + r.stderr
+
+
+def test_the_module_carries_the_interpreters_tag():
+    assert f._binding.__file__ == f._build.BINDING
+    assert f._build.BINDING.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    assert not os.path.exists(os.path.join(f._build.PKG, "_binding.so"))
