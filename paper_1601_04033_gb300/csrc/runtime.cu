@@ -10,6 +10,7 @@
 // (Eq. 1, Eq. 7 without the per-element v) is formed on the host in fp64 and
 // rounded once to fp32.
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -26,6 +27,7 @@
 #include "fasgd.h"
 #include "kernels.cuh"
 #include "message.cuh"
+#include "reach.cuh"
 #include "tensors.cuh"
 
 namespace {
@@ -71,16 +73,39 @@ std::string vformat(const char* fmt, va_list ap) {
     return buf;
 }
 
-// Whether p can be written by a copy kernel on `device`: device memory of that
-// device (not host, managed or a peer's memory), aligned to a float.
-bool local_device_floats(const void* p, int device) {
-    if (!aligned(p, 4)) return false;
+// The allocation that holds p, from the driver (looked up once: the library
+// does not link libcuda).  Without the entry point no allocation is known.
+bool find_allocation(uintptr_t p, uintptr_t* base, size_t* size) {
+    using AddressRange = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+    static const AddressRange range = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) != cudaSuccess)
+            cudaGetLastError();
+        return found == cudaDriverEntryPointSuccess ? reinterpret_cast<AddressRange>(f) : nullptr;
+    }();
+    CUdeviceptr b = 0;
+    if (range == nullptr || range(&b, size, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
+    *base = (uintptr_t)b;
+    return true;
+}
+
+// Who copies `bytes` of a server array to p.
+enum CopyRoute {
+    kCopyKernel,    // float-aligned memory of one allocation of this device
+    kCopyRuntime,   // cudaMemcpyAsync: host, managed, peer, misaligned or unknown memory
+    kCopyRefused,   // device memory that ends before the range does, as cudaMemcpyAsync refuses it
+};
+CopyRoute copy_route(const void* p, size_t bytes, int device) {
+    if (!aligned(p, 4)) return kCopyRuntime;
     cudaPointerAttributes attr;
     if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
-        cudaGetLastError();   // an unknown pointer is left to cudaMemcpyAsync
-        return false;
+        cudaGetLastError();
+        return kCopyRuntime;
     }
-    return attr.type == cudaMemoryTypeDevice && attr.device == device;
+    if (attr.type != cudaMemoryTypeDevice || attr.device != device) return kCopyRuntime;
+    const fasgd::Reach r = fasgd::reach(reinterpret_cast<uintptr_t>(p), bytes, find_allocation);
+    return r == fasgd::kReachOne ? kCopyKernel : r == fasgd::kReachShort ? kCopyRefused : kCopyRuntime;
 }
 
 // Makes h's device current for the lifetime of the guard.
@@ -1136,7 +1161,9 @@ int fasgd_pull(fasgd_t* h, float* params, int64_t* T) {
     if (params != nullptr) {
         DeviceGuard g(h->device);
         cudaError_t st = cudaSuccess;
-        if (local_device_floats(params, h->device)) {
+        const CopyRoute route = copy_route(params, (size_t)h->P * sizeof(float), h->device);
+        if (route == kCopyRefused) return h->cuda_fail(cudaErrorInvalidValue, "fasgd_pull");
+        if (route == kCopyKernel) {
             // Device memory: one kernel on the handle's stream, in order.
             fasgd::CopyArgs c;
             std::memset(&c, 0, sizeof c);
@@ -1180,7 +1207,10 @@ int fasgd_get_state(fasgd_t* h, float* theta, float* n, float* b, float* v, int6
     cudaError_t st = cudaSuccess;
     for (int i = 0; i < 4 && st == cudaSuccess; ++i) {
         if (dst[i] == nullptr) continue;
-        if (local_device_floats(dst[i], h->device)) {
+        const CopyRoute route = copy_route(dst[i], (size_t)h->P * sizeof(float), h->device);
+        if (route == kCopyRefused) {
+            st = cudaErrorInvalidValue;
+        } else if (route == kCopyKernel) {
             c.src[c.count] = src[i];
             c.dst[c.count++] = dst[i];
         } else {
