@@ -53,6 +53,12 @@ struct BlockShare {
     __host__ __device__ int32_t length(int64_t t) const { return t == 0 && piece > 0 ? piece : tile; }
 };
 
+// Blocks of a message push's pass, and float-float sums of v that it leaves: a
+// number of its own, one per SM of a GB300, so that the sums' partition, and with
+// it every bit of the statistic, is a function of P alone whatever the GPU (no
+// block waits for another, so fewer SMs take them in turns).
+constexpr int32_t kMessageBlocks = 152;
+
 // A per-message push decided before or inside its pass (FASGD rules): the pass
 // reads the decision, or takes it from the statistic's sums (message_decide)
 // where they were just formed afresh; if transmitted it applies src and copies
@@ -62,9 +68,8 @@ struct BlockShare {
 // read it).  partial == null: not a message push.
 struct PassMessage {
     const uint32_t* decided;        // the decision (1: transmitted), or null
-    const float2* fresh;            // if not decided: nblocks float-float sums of v
-    float2* partial;                // out: one sum per block of the pass
-    int32_t nblocks;
+    const float2* fresh;            // if not decided: kMessageBlocks sums of v
+    float2* partial;                // out: the sums of the new v
     float c, eps_b;
     uint32_t round_key0[10], round_key1[10];
     uint32_t client_word, n_lo, n_hi;

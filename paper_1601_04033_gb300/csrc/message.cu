@@ -7,8 +7,8 @@
 // (VSum) as it stores them, each thread its quads of the block's share in
 // order, then a fixed tree.  After any other change of v, vbar_partial_kernel
 // forms the same sums from v (same shares, same order, same bits).  The shares
-// depend on P and the number of SMs alone, so a decision does not depend on
-// which kernel formed the sums.  A decision (message_decide, one warp) adds the
+// depend on P alone (kMessageBlocks), so a decision depends neither on which
+// kernel formed the sums nor on the GPU.  A decision (message_decide, one warp) adds the
 // sums in a fixed order, forms vbar = fl32(sum / P) (ff_div_int), draws u
 // (Philox4x32-10, word 0 at counter (2^32-1, client + 2^31 * stream, n)) and
 // takes the exact Eq. 9 test.
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(32) message_decide_kernel(const __grid_constan
     pdl_wait();
     pdl_trigger();
     float vbar;
-    const uint32_t send = message_decide(a.partial, a.nblocks, a.P, a.c, a.eps_b, a.round_key0,
+    const uint32_t send = message_decide(a.partial, a.P, a.c, a.eps_b, a.round_key0,
                                          a.round_key1, a.client_word, a.n_lo, a.n_hi, &vbar);
     if (threadIdx.x == 0) {
         *a.decided = send;
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kMsgThreads) message_resolve_kernel(const __gr
     pdl_trigger();
     if (threadIdx.x < 32) {
         float vbar;
-        const uint32_t send = message_decide(a.partial, a.nblocks, a.P, a.c, a.eps_b,
+        const uint32_t send = message_decide(a.partial, a.P, a.c, a.eps_b,
                                              a.round_key0, a.round_key1, a.client_word, a.n_lo,
                                              a.n_hi, &vbar);
         if (threadIdx.x == 0) {
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kMsgThreads) message_resolve_kernel(const __gr
 }  // namespace
 
 cudaError_t launch_message_sums(const MessageArgs& a, cudaStream_t stream, int64_t* launches) {
-    const cudaError_t st = launch_pdl(vbar_partial_kernel, a.nblocks, kSumThreads, 0, stream, a);
+    const cudaError_t st = launch_pdl(vbar_partial_kernel, kMessageBlocks, kSumThreads, 0, stream, a);
     if (st == cudaSuccess) ++*launches;
     return st;
 }

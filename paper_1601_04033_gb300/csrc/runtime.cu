@@ -195,7 +195,7 @@ struct fasgd_s {
     // floats, allocated by the first message push) and the sums of v.
     float* grad_cache = nullptr;
     int64_t cache_stride = 0;
-    float2* msg_partial = nullptr;  // one sum of v per SM's share of the parameters,
+    float2* msg_partial = nullptr;  // the sums of v over the shares of a message pass,
     float2* msg_fresh = nullptr;    //   a second set (formed before a pass that leaves its own),
     uint32_t* msg_decided = nullptr;   // and the latest push's decision: one allocation
     bool msg_sums_valid = false;    // msg_partial holds the sums of the current v
@@ -301,10 +301,10 @@ struct fasgd_s {
         cudaError_t st = cudaSuccess;
         if (msg_partial == nullptr) {
             st = cudaMalloc(reinterpret_cast<void**>(&msg_partial),
-                            ((size_t)num_sms * 2 + 1) * sizeof(float2));
+                            ((size_t)fasgd::kMessageBlocks * 2 + 1) * sizeof(float2));
             if (st == cudaSuccess) {
-                msg_fresh = msg_partial + num_sms;
-                msg_decided = reinterpret_cast<uint32_t*>(msg_fresh + num_sms);
+                msg_fresh = msg_partial + fasgd::kMessageBlocks;
+                msg_decided = reinterpret_cast<uint32_t*>(msg_fresh + fasgd::kMessageBlocks);
             }
             msg_sums_valid = false;
         }
@@ -331,7 +331,6 @@ struct fasgd_s {
         a.v = v;
         a.P = P;
         a.partial = msg_partial;
-        a.nblocks = num_sms;
         a.c = c;
         a.eps_b = eps_b;
         fasgd::philox_key_schedule(seed, a.round_key0, a.round_key1);
@@ -914,7 +913,6 @@ int fasgd_apply_pending(fasgd_t* h, int32_t K) {
                     a.msg.decided = h->msg_sums_valid ? h->msg_decided : nullptr;
                     a.msg.fresh = h->msg_fresh;
                     a.msg.partial = h->msg_partial;
-                    a.msg.nblocks = m.nblocks;
                     a.msg.c = m.c;
                     a.msg.eps_b = m.eps_b;
                     std::memcpy(a.msg.round_key0, m.round_key0, sizeof a.msg.round_key0);
