@@ -103,10 +103,12 @@ def test_fetch_messages_against_oracle():
 
 @pytest.mark.parametrize("P", [5, 2048 * 3 + 129, 100_003, 300_000])
 def test_statistic_kept_by_the_dense_pass_equals_a_fresh_sum(P):
-    """After a message push the dense pass leaves the chunk sums of the new v;
+    """After a message push the dense pass leaves its blocks' sums of the new v;
     the statistic formed from them equals, bit for bit, the one formed afresh
     from v (after set_state, which discards the kept sums), and equals the
-    oracle's mean of v.  Sizes cover the dense pass's tail (P mod 2048, 128, 4)."""
+    oracle's mean of v.  Sizes within one round of tiles (152 x 2048): every
+    block has at most one piece; test_message_pass_over_rounds_of_tiles has the
+    larger ones."""
     import torch
     from paper_1601_04033_gb300 import fasgd
     w = streams.WORKLOADS["fasgd-1.29m"].replace(lam=3, R=4)
@@ -128,6 +130,70 @@ def test_statistic_kept_by_the_dense_pass_equals_a_fresh_sum(P):
         fresh = srv.message_vbar()
         assert np.float32(kept).view(np.uint32) == np.float32(fresh).view(np.uint32), (t, kept, fresh)
         assert fresh == oracle.mean_v(state[3].cpu().numpy()), (t, fresh)
+
+
+# One round of tiles is 311,296 parameters.  A piece of 3 parameters beside whole
+# tiles, short pieces and whole tiles, more tiles per block than the ring has
+# stages (5 up to 7M, 2 beyond), both sides of that switch, and more than 32
+# quads per thread (the second level of the running sums).
+@pytest.mark.parametrize("exact", [False, True])
+@pytest.mark.parametrize("variant", [oracle.FASGD, oracle.FASGD_STD])
+@pytest.mark.parametrize("P", [311_299, 700_003, 2_000_003, 6_999_999, 7_000_001, 12_000_003])
+def test_message_pass_over_rounds_of_tiles(P, variant, exact):
+    """Message pushes sent and dropped, decided by their own kernel (the sums are
+    kept) and inside the pass (another pass came between), bit for bit against
+    dense pushes of the gradient that counts: the pushed one, or the client's
+    last sent one.  The kept statistic equals a fresh one and the oracle's mean."""
+    import torch
+    from paper_1601_04033_gb300 import fasgd
+    gen = torch.Generator("cuda").manual_seed(P)
+    pool = [torch.randn(P, generator=gen, device="cuda") * 0.1 for _ in range(4)]
+    state = [torch.randn(P, generator=gen, device="cuda") * 0.1, 0.01 + 0.01 * torch.rand(P, generator=gen, device="cuda"),
+             torch.randn(P, generator=gen, device="cuda") * 0.01, 0.5 + torch.rand(P, generator=gen, device="cuda")]
+    pair = []
+    for c in (1.5, 0.0):
+        srv = fasgd.Server(P, 3, 1e-3, variant, c_push=c, seed=SEED)
+        srv.set_exact(exact)
+        srv.set_state(*state, 0)
+        pair.append(srv)
+    message, dense = pair
+    flag = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    cache = [torch.zeros(P, device="cuda")] * 3
+    seen = set()
+
+    def same_state():
+        got, want = ([torch.empty(P, device="cuda") for _ in range(4)] for _ in range(2))
+        assert message.get_state(*got) == dense.get_state(*want)
+        for name, x, y in zip("theta n b v".split(), got, want):
+            assert torch.equal(x.view(torch.int32), y.view(torch.int32)), (t, name)
+        return got
+
+    for t in range(16):
+        inside = t % 3 == 0                 # the sums were discarded: decided in the pass
+        if inside and t > 0:
+            for srv in pair:
+                srv.push(0, srv.T, pool[(t + 1) % 4])
+                srv.apply_pending(1)
+        client, g = t % 3, pool[t % 4]
+        message.push_message(client, message.T, g, sent_dev=flag)
+        message.apply_pending(1)
+        sent = int(flag.item())
+        if sent:
+            cache[client] = g
+        dense.push(client, dense.T, cache[client])
+        dense.apply_pending(1)
+        seen.add((inside, sent))
+        if t % 4 == 3:
+            same_state()
+    assert seen == {(a, b) for a in (False, True) for b in (0, 1)}, seen
+    kept = message.message_vbar()
+    got = same_state()
+    message.set_state(*got, message.T)
+    fresh = message.message_vbar()
+    assert np.float32(kept).view(np.uint32) == np.float32(fresh).view(np.uint32)
+    assert fresh == oracle.mean_v(got[3].cpu().numpy())
+    for srv in pair:
+        srv.close()
 
 
 @pytest.mark.slow
