@@ -454,28 +454,53 @@ cudaError_t launch_rule(const DenseArgs& a, int num_sms, cudaStream_t stream) {
     }
     if (a.P / kTile < kDirectTilesPerSm * num_sms) return launch_direct<RULE, ARITH>(a, num_sms, stream);
     // How many gradient slices a stage takes (CH) and how many stages: a tile's
-    // first stage holds its state and CH gradients, the others CH each, and HBM
+    // first stage holds its state and CH gradients, the others CH each.
+    //
+    // From HBM (everything the pass touches is more than L2 holds) the pass
     // streams best with some 80 to 160 KB per SM in flight, less than the
     // shared memory would hold (reads that run further ahead only push the
     // writes together).  Sweep of CH = 1, 2, 4, 8 (512 consumers; also 4, 8
     // with two blocks of 256) by 2 to 8 stages, push + apply + pull in us at
     // 25M parameters, as before (CH = K rounded up to a power of two, every
     // stage that fits; K > 8 two blocks of 256, CH = 8) -> as chosen; the same
-    // choices were best or within 1 % at 3M, 6M and 10M:
+    // choices were best or within 1 % at 8M, 10M, 12M and 50M:
     //   FASGD  K = 1: 172.6 -> 164   2: 185 -> 176     3: 201 -> 190
     //          4: 215 -> 206         5: 231 -> 217     6: 244 -> 229
     //          8: 253 -> 254         12: 316 -> 312    16: 375 (same)   32: 631 -> 601
     //   exact  3: 204 -> 190         4: 223 -> 207     5: 222 (same)
     //          6: 238 -> 232         7: 260 -> 247     8: 273     16: 494
-    //   SGD    K = 3: 103 -> 102     6: 148 -> 146     8: 182 -> 174
+    //   SGD    K = 3: 103 -> 102     5: 133.4 -> 131.6 6: 148 -> 146     8: 182 -> 174
     //          12: 242 -> 232        16: 300 -> 287    32: 531 -> 512
+    //
+    // Out of L2 latency counts instead, and more bytes in flight pay: stages of
+    // all K gradients, as many as 192 KB per SM hold, in two blocks of 256
+    // consumers (SGD: one of 512, every stage that fits).  Push + apply in us,
+    // the choice for HBM -> this one:
+    //   FASGD  K = 1: 5M 23.5 -> 20.0, 6M 33.3 -> 31.0    2: 4M 18.6 -> 16.6, 6M 38.1 -> 36.3
+    //          3: 4M 24.3 -> 21.2    4: 2.6M 13.8 -> 12.7, 4M 27.5 -> 25.2
+    //          5: 4M 31.0 -> 28.2    6: 2.6M 19.4 -> 17.4  8: 2.6M 24.0 -> 22.3
+    //   exact  K = 1: 5M 23.7 -> 20.1   2: 4M 19.8 -> 17.2   3: 4M 26.0 -> 23.1
+    //          4: 4M 28.9 -> 27.2    5: 4M 34.0 -> 32.9   (6, 7, 8: 2.6M 24.5, 27.5, 30.8 -> 24.7, 28.0, 31.7)
+    //   SGD    K = 4: 5M 14.3 -> 13.5, 6M 22.0 -> 21.0    6: 4M 17.9 -> 17.0    8: 2.6M 11.6 -> 10.3
+    // The line is at what the pass touches, a little above L2's 129 MB, where
+    // the two cross: FASGD K = 2 at 6M (144 MB) 38.1 -> 36.3, at 7M (168 MB)
+    // 43.3 -> 44.4; K = 3 at 5.5M (154 MB) 36.9 -> 36.7; SGD K = 4 at 7M
+    // (140 MB) 25.9 -> 26.8.
+    const int64_t touched = 4 * a.P * ((RULE != kRuleSgd ? 4 : 1) + a.K);
+    const bool in_l2 = touched <= (RULE != kRuleSgd ? 150'000'000 : 130'000'000);
     if constexpr (RULE == kRuleSgd) {
         if (a.K == 1) return launch_ch<RULE, ARITH, 1>(a, 5, num_sms, stream);
         if (a.K == 2) return launch_ch<RULE, ARITH, 2>(a, 5, num_sms, stream);
-        if (a.K <= 4) return launch_ch<RULE, ARITH, 4>(a, a.K == 3 ? 4 : 3, num_sms, stream);
-        if (a.K <= 8 || a.K > 14) return launch_ch<RULE, ARITH, 8>(a, 2, num_sms, stream);
+        if (a.K <= 4) return launch_ch<RULE, ARITH, 4>(a, a.K == 3 ? 4 : in_l2 ? 5 : 3, num_sms, stream);
+        if (a.K <= 8 || a.K > 14) return launch_ch<RULE, ARITH, 8>(a, a.K == 5 || (a.K <= 8 && in_l2) ? 3 : 2, num_sms, stream);
         return launch_ch<RULE, ARITH, 4>(a, 4, num_sms, stream);
     } else {
+        if (in_l2 && a.K <= (ARITH == kArithExact ? 5 : 8)) {
+            if (a.K == 1) return launch_ch<RULE, ARITH, 1, false, 256>(a, 4, num_sms, stream);
+            if (a.K == 2) return launch_ch<RULE, ARITH, 2, false, 256>(a, 4, num_sms, stream);
+            if (a.K <= 4) return launch_ch<RULE, ARITH, 4, false, 256>(a, 3, num_sms, stream);
+            return launch_ch<RULE, ARITH, 8, false, 256>(a, 2, num_sms, stream);
+        }
         if (a.K == 1) return launch_ch<RULE, ARITH, 1>(a, 2, num_sms, stream);
         if (a.K == 2) return launch_ch<RULE, ARITH, 1>(a, 3, num_sms, stream);
         if (a.K <= 4) return launch_ch<RULE, ARITH, 2>(a, 3, num_sms, stream);

@@ -1,7 +1,7 @@
 """Every form of the dense pass by K (slices per stage, stages, consumers, plain
 grid): one fused pass of K pushes equals K passes of one push bit for bit, for
 each rule and arithmetic, with ragged sizes on both sides of the plain grid's
-limit (the passes of one push are compared with the oracle elsewhere)."""
+limit and beyond L2 (the passes of one push are compared with the oracle elsewhere)."""
 
 import pytest
 
@@ -13,10 +13,10 @@ FORMS = [("sasgd", 1, False), ("fasgd", 2, False), ("fasgd exact", 2, True),
 
 
 @pytest.mark.parametrize("name,variant,exact", FORMS)
-@pytest.mark.parametrize("small", [False, True])
-def test_fused_pass_equals_single_pushes(name, variant, exact, small):
+@pytest.mark.parametrize("where", ["grid", "ring in L2", "ring from HBM"])
+def test_fused_pass_equals_single_pushes(name, variant, exact, where):
     torch, f = torch_cuda(), binding()
-    P = 300_003 if small else ring_P(70_001)
+    P = {"grid": 300_003, "ring in L2": ring_P(70_001), "ring from HBM": 16_300_003}[where]
     gen = torch.Generator(device="cuda").manual_seed(variant + 10 * exact)
     buf = torch.zeros((33, (P + 3) // 4 * 4), device="cuda")
     rows = [buf[k, :P] for k in range(33)]
