@@ -26,11 +26,13 @@
 // the 32 bits of parameters 32 l .. 32 l + 31.  Each lane then writes its set
 // bits' offsets at their ranks into shared memory (one step per kept entry
 // instead of tests per parameter: 0.46 instead of 0.69 warp instructions per
-// parameter), and consecutive lanes fetch the kept values, so that only their
-// sectors are read, and write consecutive entries.
-// Tiles of 4096, blocks of 128 threads, eight per SM (the decision of mid-sized
-// models: 256 or 512 threads): short last waves, and work for every SM from
-// 0.6M parameters on.
+// parameter at 20 % kept), and consecutive lanes fetch the kept values, so that
+// only their sectors are read, and write consecutive entries.  A warp that keeps
+// more than a third of its 1024 reads all of them, in the decision's quads, and
+// orders 128 parameters at a time (kDenseSpan).
+// Tiles of 4096, blocks of 128 threads (the decision: eight per SM, for mid-sized
+// models 256 or 512 threads; the compaction: ten, as many as hold its registers):
+// short last waves, and work for every SM from 0.6M parameters on.
 // The whole select of 25M parameters at 20 % kept: 57 -> about 46 us with the
 // scan kernel gone (exchange of four clients 1068 -> 976 us).
 //
@@ -57,6 +59,14 @@ constexpr int kSpan = 1024;
 constexpr int kThreads = kSelectTile / 32;
 constexpr int kWarps = kThreads / 32;
 constexpr unsigned kFull = 0xffffffffu;
+// Entries kept from which on a span is read whole (copy_dense_span).  The serial
+// step per kept entry and the scattered fetches behind the first 256 cost more
+// than the tests per parameter from about a third on.  The whole select, all
+// spans the sparse way -> as it is: 25M at 35 % kept 56.4 -> 53.3 us, 60 %
+// 82.2 -> 60.2, 100 % 127.5 -> 70.8 (300 MB at 6.5 TB/s behind the decision's
+// 25 us); 1.29M 8.4 -> 7.6, 11.0 -> 7.3, 18.4 -> 8.4; below 30 % kept within
+// 3 % either way.
+constexpr int kDenseSpan = 340;
 
 __device__ __forceinline__ uint32_t smem_address(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -237,22 +247,112 @@ __global__ void __launch_bounds__(kScanThreads) bfasgd_scan_kernel(const __grid_
     if (tid == kScanThreads - 1) *a.count = warp_sum[kScanThreads / 32 - 1];
 }
 
+// A span with few entries kept (below kDenseSpan): each lane writes its set bits'
+// offsets at their ranks into shared memory, and consecutive lanes fetch the kept
+// values, kHeld of them per lane ahead of the barrier behind which the place in
+// the lists is known.
+constexpr int kHeld = 8;
+struct SparseSpan {
+    float x[kHeld];
+    int o[kHeld];
+    // word: the bits of parameters 32 lane .. 32 lane + 31; incl: the entries
+    // kept up to those.
+    __device__ __forceinline__ void load(const float* src, uint32_t word, int incl, int kept, int lane,
+                                         uint16_t* off) {
+        // From the highest bit down: one step per kept entry.
+        for (int r = incl - 1; word != 0; --r) {
+            const int b = 31 - __clz((int)word);
+            off[r] = (uint16_t)(32 * lane + b);
+            word ^= 1u << b;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < kHeld; ++i) {
+            const int k = lane + 32 * i;
+            if (k < kept) {
+                o[i] = off[k];
+                x[i] = __ldcs(src + o[i]);
+            }
+        }
+    }
+    __device__ __forceinline__ void store(const SelectArgs& a, int kept, int64_t start, int lane,
+                                          const uint16_t* off, int32_t out) const {
+#pragma unroll
+        for (int i = 0; i < kHeld; ++i) {
+            const int k = lane + 32 * i;
+            if (k < kept) {
+                a.idx[out + k] = (int32_t)start + o[i];
+                a.val[out + k] = x[i];
+            }
+        }
+        for (int k = lane + 32 * kHeld; k < kept; k += 32) {
+            const int p = off[k];
+            a.idx[out + k] = (int32_t)start + p;
+            a.val[out + k] = __ldcs(a.values + start + p);
+        }
+    }
+};
+
+// A span with many: every value is read, in the quads that the lane's bits are
+// of (nibble it: quad 32 it + lane), and each pass of 128 parameters puts its
+// kept entries in order in shared memory (two passes' room: one wait per pass)
+// for coalesced stores.
+__device__ __forceinline__ void copy_dense_span(const SelectArgs& a, uint32_t bits, int64_t start, int lane,
+                                                uint2* stage, int32_t out) {
+    // Kept entries per nibble, then their running sums over the lanes, four
+    // passes to a word (a pass keeps 128 at most): even passes, odd passes.
+    uint32_t n = bits - ((bits >> 1) & 0x55555555u);
+    n = (n & 0x33333333u) + ((n >> 2) & 0x33333333u);
+    uint32_t even = n & 0x0f0f0f0fu, odd = (n >> 4) & 0x0f0f0f0fu;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t e = __shfl_up_sync(kFull, even, d), o = __shfl_up_sync(kFull, odd, d);
+        if (lane >= d) {
+            even += e;
+            odd += o;
+        }
+    }
+    constexpr int kAtOnce = 4;   // quads per lane in flight: eight would cost the kernel a third of its warps
+    float4 q[kAtOnce];
+    const uint32_t all_even = __shfl_sync(kFull, even, 31), all_odd = __shfl_sync(kFull, odd, 31);
+#pragma unroll
+    for (int it = 0; it < 8; ++it) {
+        if (it % kAtOnce == 0) load_quads(q, a.values, start + 128 * it, a.P, lane);
+        const int sh = 8 * (it >> 1);
+        const int total = (int)(((it & 1) ? all_odd : all_even) >> sh & 0xffu);
+        int r = (int)(((it & 1) ? odd : even) >> sh & 0xffu) - (int)(n >> (4 * it) & 0xfu);
+        const uint32_t e = (uint32_t)start + 128 * it + 4 * lane;   // P < 2^31
+        const float4 v = q[it % kAtOnce];
+        const uint32_t x[4] = {__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w)};
+        uint2* s = stage + 128 * (it & 1);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (bits >> (4 * it + j) & 1u) s[r++] = make_uint2(e + j, x[j]);
+        __syncwarp();
+        for (int k = lane; k < total; k += 32) {
+            const uint2 y = s[k];
+            a.idx[out + k] = (int32_t)y.x;
+            a.val[out + k] = __uint_as_float(y.y);
+        }
+        out += total;
+    }
+}
+
 // SCANNED: tile_base holds the sums (bfasgd_scan_kernel), else the block adds
 // the counts before its tile.
 template <bool SCANNED>
-__global__ void __launch_bounds__(kThreads, 8) bfasgd_compact_kernel(const __grid_constant__ SelectArgs a) {
-    __shared__ uint16_t s_off[kWarps][kSpan];
+__global__ void __launch_bounds__(kThreads, 10) bfasgd_compact_kernel(const __grid_constant__ SelectArgs a) {
+    __shared__ __align__(16) unsigned char s_span[kWarps][2 * kSpan];
     __shared__ int32_t warp_cnt[kWarps], warp_sum[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint16_t* off = s_off[warp];
     const int64_t start = (int64_t)blockIdx.x * kSelectTile + warp * kSpan;
     pdl_wait();
     pdl_trigger();
     const uint32_t bits = a.mask[(start >> 5) + lane];
-    int64_t tile_out = 0;
+    int32_t tile_out = 0;   // places in the lists are below P < 2^31
     int32_t before = 0;
     if (SCANNED) {
-        tile_out = a.tile_base[blockIdx.x];
+        tile_out = (int32_t)a.tile_base[blockIdx.x];
     } else {
         // Eight counts per load; the last load's own and later ones are left out.
         for (int t = 8 * threadIdx.x; t < (int)blockIdx.x; t += 8 * kThreads) {
@@ -266,9 +366,8 @@ __global__ void __launch_bounds__(kThreads, 8) bfasgd_compact_kernel(const __gri
             }
         }
     }
-    uint32_t word = lane_word(bits, lane);
-    const int n = __popc(word);
-    int incl = n;
+    const uint32_t word = lane_word(bits, lane);
+    int incl = __popc(word);
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
         const int y = __shfl_up_sync(kFull, incl, d);
@@ -279,27 +378,11 @@ __global__ void __launch_bounds__(kThreads, 8) bfasgd_compact_kernel(const __gri
         before = (int32_t)__reduce_add_sync(kFull, (uint32_t)before);
         if (lane == 0) warp_sum[warp] = before;
     }
-    // From the highest bit down: one step per kept entry.
-    for (int r = incl - 1; word != 0; --r) {
-        const int b = 31 - __clz((int)word);
-        off[r] = (uint16_t)(32 * lane + b);
-        word ^= 1u << b;
-    }
-    __syncwarp();
-    const int mine = __shfl_sync(kFull, incl, 31);
-    // The kept values, in the order of the list.
-    const float* src = a.values + start;
-    constexpr int kHeld = 8;
-    float x[kHeld];
-    int o[kHeld];
-#pragma unroll
-    for (int i = 0; i < kHeld; ++i) {
-        const int k = lane + 32 * i;
-        if (k < mine) {
-            o[i] = off[k];
-            x[i] = __ldcs(src + o[i]);
-        }
-    }
+    const int kept = __shfl_sync(kFull, incl, 31);
+    const bool sparse = kept < kDenseSpan;   // the whole warp's
+    uint16_t* off = reinterpret_cast<uint16_t*>(s_span[warp]);
+    SparseSpan span;
+    if (sparse) span.load(a.values + start, word, incl, kept, lane, off);
     __syncthreads();
     int32_t ahead = 0;
 #pragma unroll
@@ -307,23 +390,12 @@ __global__ void __launch_bounds__(kThreads, 8) bfasgd_compact_kernel(const __gri
         if (!SCANNED) ahead += warp_sum[w];
         if (w < warp) ahead += warp_cnt[w];
     }
-    const int64_t out = tile_out + ahead;
-    int32_t* idx_out = a.idx + out;
-    float* val_out = a.val + out;
-#pragma unroll
-    for (int i = 0; i < kHeld; ++i) {
-        const int k = lane + 32 * i;
-        if (k < mine) {
-            idx_out[k] = (int32_t)start + o[i];
-            val_out[k] = x[i];
-        }
-    }
-    for (int k = lane + 32 * kHeld; k < mine; k += 32) {
-        const int p = off[k];
-        idx_out[k] = (int32_t)start + p;
-        val_out[k] = __ldcs(src + p);
-    }
-    if (!SCANNED && blockIdx.x == gridDim.x - 1 && warp == kWarps - 1 && lane == 0) *a.count = out + mine;
+    const int32_t out = tile_out + ahead;
+    if (sparse)
+        span.store(a, kept, start, lane, off, out);
+    else
+        copy_dense_span(a, bits, start, lane, reinterpret_cast<uint2*>(s_span[warp]), out);
+    if (!SCANNED && blockIdx.x == gridDim.x - 1 && warp == kWarps - 1 && lane == 0) *a.count = (int64_t)out + kept;
 }
 
 }  // namespace
