@@ -107,6 +107,8 @@ struct SparseArgs {
     float coef;
     StatParams sp;
     int32_t* err;              // device error flags (bit 0: count, bit 1: index, bit 2: order)
+    int64_t half_below, quarter_below;   // set by the launch: lists shorter than these take
+                                         // half, a quarter of the warps
 };
 
 // Parameters per tile of the select kernels, and the bit mask words a tile

@@ -15,9 +15,7 @@
 // TB/s), and by latency for small models: with the first list entries asked for
 // beside the count and two entries per thread instead of four, four exchanges
 // take 107 instead of 112 us at 1.29M, 154 instead of 177 at 3M, 271 instead of
-// 277 at 6M.
-
-#include <atomic>
+// 277 at 6M (launch_rule has the forms and their figures).
 
 #include "kernels.cuh"
 #include "pdl.cuh"
@@ -28,13 +26,14 @@ namespace {
 
 constexpr int kSparseThreads = 256;
 
-// AHEAD: the first step's list entries are loaded beside the count.
-template <int RULE, bool EXACT, int kUnroll, bool AHEAD>
-__global__ void __launch_bounds__(kSparseThreads, !AHEAD ? 1 : EXACT ? 6 : 8) fasgd_sparse_kernel(const __grid_constant__ SparseArgs a) {
+// AHEAD: the first step's list entries are loaded beside the count.  BLOCKS: blocks
+// per SM that the registers are held to.
+template <int RULE, bool EXACT, int kUnroll, bool AHEAD, int BLOCKS>
+__global__ void __launch_bounds__(kSparseThreads, BLOCKS) fasgd_sparse_kernel(const __grid_constant__ SparseArgs a) {
     constexpr bool FAS = RULE != kRuleSgd;
     const int lane = threadIdx.x & 31;
-    const int64_t warp_id = ((int64_t)blockIdx.x * kSparseThreads + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * kSparseThreads) >> 5;
+    int64_t warp_id = ((int64_t)blockIdx.x * kSparseThreads + threadIdx.x) >> 5;
+    int64_t nwarps = ((int64_t)gridDim.x * kSparseThreads) >> 5;
     pdl_wait();
     pdl_trigger();
     int64_t count = a.count_max;
@@ -53,12 +52,20 @@ __global__ void __launch_bounds__(kSparseThreads, !AHEAD ? 1 : EXACT ? 6 : 8) fa
             }
         }
     };
-    const int64_t first = warp_id * (32 * kUnroll);
-    if (AHEAD) load(first, a.count_max);
+    if (AHEAD) load(warp_id * (32 * kUnroll), a.count_max);
     if (a.count_dev != nullptr && (count < 0 || count > a.count_max)) {
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.err, 1);
         count = count < 0 ? 0 : a.count_max;
     }
+    if constexpr (!AHEAD) {
+        if (count < a.half_below) {   // half or a quarter of each block's warps
+            const int part = count < a.quarter_below ? 4 : 2;
+            if (threadIdx.x >= kSparseThreads / part) return;
+            warp_id = ((int64_t)blockIdx.x * (kSparseThreads / part) + threadIdx.x) >> 5;
+            nwarps /= part;
+        }
+    }
+    const int64_t first = warp_id * (32 * kUnroll);
     for (int64_t base = first; base < count; base += nwarps * (32 * kUnroll)) {
         bool ok[kUnroll];
         if (!AHEAD || base != first) load(base, count);
@@ -105,37 +112,50 @@ __global__ void __launch_bounds__(kSparseThreads, !AHEAD ? 1 : EXACT ? 6 : 8) fa
     }
 }
 
-template <int RULE, bool EXACT, int kUnroll, bool AHEAD>
+template <int RULE, bool EXACT, int kUnroll, bool AHEAD, int BLOCKS>
 cudaError_t launch_form(const SparseArgs& a, int num_sms, cudaStream_t stream) {
-    // Resident blocks per SM, looked up once (the grid is only capped by it).
-    static std::atomic<int> cached{0};
-    int blocks_per_sm = cached.load(std::memory_order_relaxed);
-    if (blocks_per_sm == 0) {
-        cudaError_t st = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &blocks_per_sm, fasgd_sparse_kernel<RULE, EXACT, kUnroll, AHEAD>, kSparseThreads, 0);
-        if (st != cudaSuccess) return st;
-        if (blocks_per_sm < 1) blocks_per_sm = 1;
-        cached.store(blocks_per_sm, std::memory_order_relaxed);
-    }
     // Enough warps for the host-side bound on the count, at most one full wave.
     const int64_t per_block = (int64_t)kSparseThreads * kUnroll;
     int64_t want = (a.count_max + per_block - 1) / per_block;
-    const int64_t cap = (int64_t)num_sms * blocks_per_sm;
+    const int64_t cap = (int64_t)num_sms * BLOCKS;
     if (want > cap) want = cap;
     if (want < 1) want = 1;
-    return launch_pdl(fasgd_sparse_kernel<RULE, EXACT, kUnroll, AHEAD>, (unsigned)want, kSparseThreads, 0, stream, a);
+    return launch_pdl(fasgd_sparse_kernel<RULE, EXACT, kUnroll, AHEAD, BLOCKS>, (unsigned)want, kSparseThreads, 0, stream, a);
 }
 
-// Models up to 10M parameters: two entries per thread, the first step's ahead of
-// the count, as many warps as fit (latency shows there).  Larger ones: four after
-// it and registers to hold them, two blocks per SM: with fewer bytes in flight
-// HBM serves the scattered sectors faster (four exchanges at 25M: 957 us against
-// 980 with the small form and 975 with six blocks; 7M 319 against 313; 12M 499
-// against 502; 16M 640 against 650).
+// FASGD rules, up to 7M entries at most: two per thread, the first step's ahead of
+// the count, as many warps as fit (latency shows there).  Beyond: four per thread,
+// four blocks per SM, and of each block's warps all, half or a quarter, by the
+// list's density.  Scattered sectors HBM serves faster with fewer bytes in flight
+// (under 45 % kept half the warps, under 14 % a quarter), a dense list, whose
+// gathers are coalesced, needs all of them.  (Part of each block, since the first
+// blocks of a larger grid do not spread over the SMs: 20 % at 25M 138 us so.)  One
+// apply in us, the forms it replaces -- four per thread and 48 registers at every
+// size, then the small form up to 10M and 83 registers beyond, which left two
+// blocks per SM at any density -- and this:
+//   kept        5 %                  20 %                  60 %                  100 %
+//   25M    111.6, 106.5, 93.1   127.6, 123.2, 124.1   150.5, 168.5, 148.2   160.8, 196.8, 153.2
+//   12M     46.1,  48.2, 44.1    66.2,  61.2,  61.3    74.7,  82.6,  72.7    79.5,  96.8,  76.8
+//   9M      26.4,  28.0, 24.4    44.4,  45.1,  44.7    56.4,  55.7,  55.1    60.5,  57.0,  57.4
+// At 6M the two forms are within 4 % (10 % kept 17.4 small, 18.1 large; 60 %
+// 31.6, 30.9).
+// ASGD/SASGD gather one array: four per thread, five blocks per SM, all the warps
+// (25M: half would take 41 against 34 us at 20 %, 118 against 68 at 100 %) but for
+// large models under 6 % kept (15.5 -> 13.3 at 5 %); at 3M and 6M, all kept, 5.6
+// and 10.0 against 7.1 and 13.5 in the small form.
 template <int RULE, bool EXACT>
-cudaError_t launch_rule(const SparseArgs& a, int num_sms, cudaStream_t stream) {
-    return a.count_max <= 10'000'000 ? launch_form<RULE, EXACT, 2, true>(a, num_sms, stream)
-                                     : launch_form<RULE, EXACT, 4, false>(a, num_sms, stream);
+cudaError_t launch_rule(SparseArgs a, int num_sms, cudaStream_t stream) {
+    const bool large = a.count_max > 7'000'000;
+    if constexpr (RULE == kRuleSgd) {
+        a.half_below = large ? a.P / 16 : 0;
+        a.quarter_below = 0;
+        return launch_form<RULE, EXACT, 4, false, 5>(a, num_sms, stream);
+    } else {
+        a.half_below = a.P / 20 * 9;
+        a.quarter_below = a.P / 7;
+        return large ? launch_form<RULE, EXACT, 4, false, 4>(a, num_sms, stream)
+                     : launch_form<RULE, EXACT, 2, true, EXACT ? 6 : 8>(a, num_sms, stream);
+    }
 }
 
 constexpr int kScatterUnroll = 8;

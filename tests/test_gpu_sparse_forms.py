@@ -1,5 +1,6 @@
-"""The sparse apply on both sides of the switch between its two forms (10M
-parameters of host-side bound) and at counts around its steps, against the
+"""The sparse apply on both sides of the switch between its forms (7M
+parameters of host-side bound), at counts around its steps and around the
+densities from which half and all of the large form's warps work, against the
 oracle on the listed parameters; lists without a device count, short and empty."""
 
 import numpy as np
@@ -9,7 +10,11 @@ import oracle
 from gpu_util import ATOL, RTOL, binding, torch_cuda
 
 pytestmark = pytest.mark.gpu
-SWITCH = 10_000_000
+SWITCH = 7_000_000
+COUNTS = ((0, True), (1, False), (31, True), (33, False), (63, True), (257, True), (60_001, False),
+          (700_003, True), (2_600_001, True))
+# Large form: a sixteenth (SASGD), a seventh, nine twentieths of P, and all of it.
+LINES = tuple((m, True) for m in (437_499, 437_500, 999_999, 1_000_000, 3_149_999, 3_150_000, SWITCH + 1))
 
 
 @pytest.mark.parametrize("variant,exact", [(oracle.FASGD, False), (oracle.FASGD, True),
@@ -25,8 +30,7 @@ def test_both_forms(P, variant, exact):
              rng.random(P, dtype=np.float32) * np.float32(50) + np.float32(1)]
     srv.set_state(*[torch.from_numpy(x).cuda() for x in state], 0)
     out = [torch.empty(P, device="cuda") for _ in range(4)]
-    for m, device_count in ((0, True), (1, False), (31, True), (33, False), (63, True), (257, True),
-                            (60_001, False), (700_003, True), (2_600_001, True)):
+    for m, device_count in COUNTS + (LINES if P > SWITCH else ()):
         keep = np.sort(rng.choice(P, m, replace=False)).astype(np.int32)
         g = (rng.standard_normal(m) * 0.05).astype(np.float32)
         idx = torch.zeros(P if device_count else max(m, 1), dtype=torch.int32, device="cuda")
