@@ -184,7 +184,7 @@ fasgd_dense_kernel(const __grid_constant__ DenseArgs a, const Ring ring) {
             __shared__ uint32_t s_send;
             if (warp == 0) {
                 float vbar;
-                const uint32_t d = message_decide(a.msg.fresh, a.P, a.msg.c, a.msg.eps_b,
+                const uint32_t d = message_decide(a.msg.fresh, a.msg.nblocks, a.P, a.msg.c, a.msg.eps_b,
                                                   a.msg.round_key0, a.msg.round_key1, a.msg.client_word,
                                                   a.msg.n_lo, a.msg.n_hi, &vbar);
                 if (lane == 0) {

@@ -70,6 +70,7 @@ struct PassMessage {
     const uint32_t* decided;        // the decision (1: transmitted), or null
     const float2* fresh;            // if not decided: kMessageBlocks sums of v
     float2* partial;                // out: the sums of the new v
+    int32_t nblocks;                // kMessageBlocks
     float c, eps_b;
     uint32_t round_key0[10], round_key1[10];
     uint32_t client_word, n_lo, n_hi;

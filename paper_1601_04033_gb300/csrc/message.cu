@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(32) message_decide_kernel(const __grid_constan
     pdl_wait();
     pdl_trigger();
     float vbar;
-    const uint32_t send = message_decide(a.partial, a.P, a.c, a.eps_b, a.round_key0,
+    const uint32_t send = message_decide(a.partial, a.nblocks, a.P, a.c, a.eps_b, a.round_key0,
                                          a.round_key1, a.client_word, a.n_lo, a.n_hi, &vbar);
     if (threadIdx.x == 0) {
         *a.decided = send;
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kMsgThreads) message_resolve_kernel(const __gr
     pdl_trigger();
     if (threadIdx.x < 32) {
         float vbar;
-        const uint32_t send = message_decide(a.partial, a.P, a.c, a.eps_b,
+        const uint32_t send = message_decide(a.partial, a.nblocks, a.P, a.c, a.eps_b,
                                              a.round_key0, a.round_key1, a.client_word, a.n_lo,
                                              a.n_hi, &vbar);
         if (threadIdx.x == 0) {

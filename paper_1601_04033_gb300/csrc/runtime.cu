@@ -331,6 +331,7 @@ struct fasgd_s {
         a.v = v;
         a.P = P;
         a.partial = msg_partial;
+        a.nblocks = fasgd::kMessageBlocks;
         a.c = c;
         a.eps_b = eps_b;
         fasgd::philox_key_schedule(seed, a.round_key0, a.round_key1);
@@ -913,6 +914,7 @@ int fasgd_apply_pending(fasgd_t* h, int32_t K) {
                     a.msg.decided = h->msg_sums_valid ? h->msg_decided : nullptr;
                     a.msg.fresh = h->msg_fresh;
                     a.msg.partial = h->msg_partial;
+                    a.msg.nblocks = m.nblocks;
                     a.msg.c = m.c;
                     a.msg.eps_b = m.eps_b;
                     std::memcpy(a.msg.round_key0, m.round_key0, sizeof a.msg.round_key0);
