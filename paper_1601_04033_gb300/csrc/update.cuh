@@ -147,30 +147,51 @@ template <int ARITH> struct Guard {
     __device__ __forceinline__ bool ok() const { return true; }
 };
 
-// fasgd_update_exact on two parameters, the same bits.  CUDA's own square
-// root and division are correctly rounded over the whole fp32 range and cost
-// about 80 issue slots per element-push here, which made the exact pass
-// issue-bound (K = 8 at 25M parameters: 427 us, 55 % of the copy bandwidth).
-// Inside the range above, which every finite training run keeps to, the
-// hardware approximations refined by fused multiply-adds are correctly rounded
-// as well (Markstein, IBM J. Res. Dev. 34(1), 1990: the residual of an almost
-// rounded root or quotient is exact in one fused multiply-add, and one
-// correction by a rounded reciprocal then rounds correctly):
+// Square root, reciprocal and quotient of pairs.  CUDA's own square root and
+// division are correctly rounded over the whole fp32 range and cost about 80
+// issue slots per element-push here, which made the exact pass issue-bound
+// (K = 8 at 25M parameters: 427 us, 55 % of the copy bandwidth).  Inside the
+// range above, which every finite training run keeps to, the hardware
+// approximations refined by fused multiply-adds are correctly rounded as well
+// (Markstein, IBM J. Res. Dev. 34(1), 1990: the residual of an almost rounded
+// root or quotient is exact in one fused multiply-add, and one correction by a
+// rounded reciprocal then rounds correctly):
 //   root:        s = rad y, y ~ rad^-1/2;   s + (rad - s^2) y / 2
 //   reciprocal:  z ~ 1 / x;                 z + (1 - x z) z
 //   quotient:    q = a z, z = fl(1/v);      twice q + (a - v q) z (the first
 //                makes q faithful, the second rounds it).
-// The quotient is formed as -q, which keeps the sign of a zero a.  Root
-// and reciprocal were compared with __fsqrt_rn and __fdiv_rn for every fp32
-// value of the range, the quotient on 4e10 pairs (random, near midpoints,
-// mantissas at both ends): no difference; the approximation of a negated value
-// is the negated approximation, for every value of the range as well.  25M, K = 8
-// / 16, push + apply + pull: 464 us with CUDA's functions (K = 8), 282 / 517 with
-// the negations as operations of their own, 273 / 494 now.
+// Reciprocal and quotient come negated (the sign is free at the approximation's
+// input), which keeps the sign of a zero a.  tests/test_gpu_exact_sweep.py holds
+// these three functions to CUDA's: root and reciprocal for every fp32 value of
+// the range, the quotient on 4e10 pairs (random, near midpoints, mantissas at
+// both ends).
+__device__ __forceinline__ Pair root2(Pair rad, Pair minus_rad) {
+    float x, y;
+    unpack(rad, x, y);
+    const Pair inv = pair(rsqrt_approx<true>(x), rsqrt_approx<true>(y));
+    const Pair s = mul2(rad, inv);
+    return fma2(fma2(s, s, minus_rad), mul2(inv, pair(-0.5f, -0.5f)), s);
+}
+__device__ __forceinline__ Pair minus_reciprocal2(Pair x) {
+    float a, b;
+    unpack(x, a, b);
+    const Pair w = pair(rcp_approx<true>(-a), rcp_approx<true>(-b));
+    return fma2(fma2(x, w, pair(1.f, 1.f)), w, w);
+}
+// -(a / v), given the correctly rounded -(1 / v).
+__device__ __forceinline__ Pair minus_quotient2(Pair a, Pair v, Pair minus_z) {
+    Pair minus_q = mul2(a, minus_z);
+    minus_q = fma2(fma2(v, minus_q, a), minus_z, minus_q);
+    return fma2(fma2(v, minus_q, a), minus_z, minus_q);
+}
+
+// fasgd_update_exact on two parameters, the same bits.  25M, K = 8 / 16, push +
+// apply + pull: 464 us with CUDA's functions (K = 8), 282 / 517 with the negations
+// as operations of their own, 273 / 494 now.
 template <bool STD, class G>
 __device__ __forceinline__ void exact_update2(Pair& theta, Pair& n, Pair& b, Pair& v, Pair g, float coef,
                                               const StatParams& sp, G& guard) {
-    const Pair minus1 = pair(-1.f, -1.f), one = pair(1.f, 1.f);
+    const Pair minus1 = pair(-1.f, -1.f);
     const Pair gamma = pair(sp.gamma, sp.gamma), rest = pair(sp.one_m_gamma, sp.one_m_gamma);
     n = add2(product2(gamma, n, sp), product2(rest, mul2(g, g), sp));
     b = add2(product2(gamma, b, sp), product2(rest, g, sp));
@@ -181,32 +202,17 @@ __device__ __forceinline__ void exact_update2(Pair& theta, Pair& n, Pair& b, Pai
     const Pair minus_rad = fma2(var, minus1, pair(-sp.eps, -sp.eps));
     unpack(rad, x, y);
     guard.see_rad(x, y);
-    const Pair inv = pair(rsqrt_approx<true>(x), rsqrt_approx<true>(y));
-    const Pair s = mul2(rad, inv);
-    const Pair root = fma2(fma2(s, s, minus_rad), mul2(inv, pair(-0.5f, -0.5f)), s);
-    // v' = beta v + (1 - beta) r.  The reciprocals are those of negated values
-    // (the sign is free at the approximation's input), so r and z come negated.
-    Pair step;
-    if (STD) {
-        step = product2(pair(sp.one_m_beta, sp.one_m_beta), root, sp);
-    } else {
-        unpack(root, x, y);
-        const Pair w = pair(rcp_approx<true>(-x), rcp_approx<true>(-y));
-        const Pair minus_r = fma2(fma2(root, w, one), w, w);
-        step = product2(pair(-sp.one_m_beta, -sp.one_m_beta), minus_r, sp);
-    }
+    const Pair root = root2(rad, minus_rad);
+    // v' = beta v + (1 - beta) r.
+    const Pair step = STD ? product2(pair(sp.one_m_beta, sp.one_m_beta), root, sp)
+                          : product2(pair(-sp.one_m_beta, -sp.one_m_beta), minus_reciprocal2(root), sp);
     v = add2(product2(pair(sp.beta, sp.beta), v, sp), step);
     unpack(v, x, y);
     guard.see_v(x, y);
-    const Pair w = pair(rcp_approx<true>(-x), rcp_approx<true>(-y));
-    const Pair minus_z = fma2(fma2(v, w, one), w, w);
     const Pair a = mul2(pair(coef, coef), g);
     unpack(a, x, y);
     guard.see_a(x, y);
-    Pair minus_q = mul2(a, minus_z);
-    minus_q = fma2(fma2(v, minus_q, a), minus_z, minus_q);
-    minus_q = fma2(fma2(v, minus_q, a), minus_z, minus_q);
-    theta = add2(theta, minus_q);
+    theta = add2(theta, minus_quotient2(a, v, minus_reciprocal2(v)));
 }
 
 // Arithmetic of a pass: hardware approximations (subnormal-preserving or
