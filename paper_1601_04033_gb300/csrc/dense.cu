@@ -482,6 +482,8 @@ cudaError_t launch_rule(const DenseArgs& a, int num_sms, cudaStream_t stream) {
     //   exact  K = 1: 5M 23.7 -> 20.1   2: 4M 19.8 -> 17.2   3: 4M 26.0 -> 23.1
     //          4: 4M 28.9 -> 27.2    5: 4M 34.0 -> 32.9   (6, 7, 8: 2.6M 24.5, 27.5, 30.8 -> 24.7, 28.0, 31.7)
     //   SGD    K = 4: 5M 14.3 -> 13.5, 6M 22.0 -> 21.0    6: 4M 17.9 -> 17.0    8: 2.6M 11.6 -> 10.3
+    //          K = 1 alone the same, behind other kernels less: with a pull 8M 19.2 -> 17.0,
+    //          dropped message pushes at 12M 23.7 -> 18.3, with a budget push at 5M 21.5 -> 19.7
     // The line is at what the pass touches, a little above L2's 129 MB, where
     // the two cross: FASGD K = 2 at 6M (144 MB) 38.1 -> 36.3, at 7M (168 MB)
     // 43.3 -> 44.4; K = 3 at 5.5M (154 MB) 36.9 -> 36.7; SGD K = 4 at 7M
@@ -489,7 +491,7 @@ cudaError_t launch_rule(const DenseArgs& a, int num_sms, cudaStream_t stream) {
     const int64_t touched = 4 * a.P * ((RULE != kRuleSgd ? 4 : 1) + a.K);
     const bool in_l2 = touched <= (RULE != kRuleSgd ? 150'000'000 : 130'000'000);
     if constexpr (RULE == kRuleSgd) {
-        if (a.K == 1) return launch_ch<RULE, ARITH, 1>(a, 5, num_sms, stream);
+        if (a.K == 1) return launch_ch<RULE, ARITH, 1>(a, in_l2 ? 8 : 5, num_sms, stream);
         if (a.K == 2) return launch_ch<RULE, ARITH, 2>(a, 5, num_sms, stream);
         if (a.K <= 4) return launch_ch<RULE, ARITH, 4>(a, a.K == 3 ? 4 : in_l2 ? 5 : 3, num_sms, stream);
         if (a.K <= 8 || a.K > 14) return launch_ch<RULE, ARITH, 8>(a, a.K == 5 || (a.K <= 8 && in_l2) ? 3 : 2, num_sms, stream);
