@@ -264,7 +264,8 @@ FASGD_API int bfasgd_fetch_apply(int64_t P, float* theta_client, const int32_t* 
  * bfasgd_push_message -- the paper's literal B-FASGD push (Sec. 2.3): one
  * decision for the whole message.  When the push is applied (in arrival
  * order, by fasgd_apply_pending), the server forms vbar = the mean of v over
- * all P parameters (a compensated sum in a fixed order, rounded once to fp32), draws u
+ * all P parameters (a compensated sum in an order that P alone fixes, whatever
+ * the GPU, rounded once to fp32), draws u
  * (Philox4x32-10 word 0 at counter (2^32-1, client, n, n >> 32), key = seed,
  * n = the client's push count, which then advances) and transmits iff Eq. 9
  * holds: u / 2^24 < 1 / (1 + c_push / (vbar + eps_b)), decided exactly in
@@ -296,7 +297,7 @@ FASGD_API int bfasgd_fetch_message(fasgd_t* h, int32_t client, float* theta_clie
 /*
  * bfasgd_message_vbar -- the statistic the per-message decision would use
  * now: vbar = the mean of the server's v over all P parameters (a
- * compensated sum in a fixed order, rounded once to fp32), written to
+ * compensated sum in an order that P alone fixes, rounded once to fp32), written to
  * vbar_dev (device float) on the handle's stream.  No draw is consumed and
  * no counter advances.  Errors: EINVAL, ENOMEM, ECUDA.
  */
@@ -371,7 +372,8 @@ FASGD_API int bfasgd_fetch_budget(fasgd_t* h, int32_t client, float* theta_clien
  * handed back to a client).  The copy is ordered after earlier work on the
  * handle's stream and later work on that stream waits for it (a copy to host
  * memory runs on an internal stream beside pending host-push copies).
- * Pending pushes are not applied.
+ * Pending pushes are not applied.  Device memory that ends before P values do
+ * is refused (ECUDA).
  * Either output may be NULL.  Errors: EINVAL, ECUDA.
  */
 FASGD_API int fasgd_pull(fasgd_t* h, float* params, int64_t* T);
@@ -379,7 +381,8 @@ FASGD_API int fasgd_pull(fasgd_t* h, float* params, int64_t* T);
 /*
  * fasgd_get_state / fasgd_set_state -- checkpoint and restore theta, n, b, v
  * (P fp32 each; host or device; any may be NULL to skip it) and T.
- * Both require an empty queue.  get_state blocks until the copies are done.
+ * Both require an empty queue.  get_state blocks until the copies are done, and
+ * refuses device memory that ends before P values do (ECUDA).
  * Errors: EINVAL, EAGAIN (pushes pending), ECUDA.
  */
 FASGD_API int fasgd_get_state(fasgd_t* h, float* theta, float* n, float* b, float* v, int64_t* T);

@@ -405,10 +405,11 @@ void select_key_schedule(SelectArgs& a, uint64_t seed) {
 }
 
 cudaError_t launch_select(const SelectArgs& a, cudaStream_t stream, int64_t* launches) {
-    // Quads per lane: with about two to seven tiles per SM shorter chains of
-    // draws per warp (and more warps) pay; below that a tile's 16 warps would
-    // crowd one SM while others idle, above it the SMs are full anyway.  Four
-    // exchanges with 2 / 4 / 8, us: 600,000 78 / 72 / 72, 800,000 83 / 84 / 80,
+    // Quads per lane: from 1.4 to 7.2 tiles per SM shorter chains of draws per
+    // warp (and more warps) pay; below that a tile's 16 warps would crowd one SM
+    // while others idle, above it the SMs are full anyway.  Four exchanges
+    // without a pull, one after the other on the same buffers, with 2 / 4 / 8
+    // (the compaction then as it was before kDenseSpan), us: 600,000 78 / 72 / 72, 800,000 83 / 84 / 80,
     // 1.0M 88 / 92 / 93, 1.29M 90 / 101 / 107, 1.6M 109 / 109 / 119, 2M 122 /
     // 117 / 127, 4M 207 / 196 / 196, 8M 372 / 356 / 350.
     cudaError_t st = a.P > 850'000 && a.P <= 1'500'000     ? launch_decide<2>(a, stream)
