@@ -11,7 +11,7 @@
 // coalesced and kUnroll gathers per array are in flight per thread.
 //
 // Bound by HBM at the granularity of sectors: at 20 % kept almost every sector
-// of theta, n, b, v is read and most are written (25M: 725 MB in about 117 us, 6.2
+// of theta, n, b, v is read and most are written (25M: 721 MB in about 120 us, 6.0
 // TB/s), and by latency for small models: with the first list entries asked for
 // beside the count and two entries per thread instead of four, four exchanges
 // take 107 instead of 112 us at 1.29M, 154 instead of 177 at 3M, 271 instead of
