@@ -137,11 +137,17 @@ __device__ __forceinline__ Pair product2(Pair a, Pair b, const StatParams& sp) {
 }
 
 // What the pushes of a pass saw, kept while they are applied: whether the
-// chains of exact_update2 were correctly rounded throughout.  That holds for
-// rad in [2^-100, 2^100], v in [2^-60, 2^60] and a = fl(coef g) zero or of
-// magnitude in [2^-60, 2^60]: no intermediate is then subnormal and no
-// residual rounded.  NaN fails.  One add-and-compare instruction per bound,
-// and no branch among the pushes: a pass looks once, at its end, and forms
+// chains of exact_update2 gave the correctly rounded sequence throughout.  That
+// holds for rad in [2^-100, 2^100], v in [2^-60, 2^60] and a quotient q = a / v,
+// a = fl(coef g), that is zero or of magnitude in [2^-66, 2^80]: a and q are then
+// normal, no intermediate is subnormal and no residual rounded.  A smaller q does
+// no harm either where |theta| is 2^-40 or more: half the gap to its neighbours is
+// at least 2^-65, so theta stays as it is whatever q rounds to.  Gradients far
+// below their neighbours, as a saturated softmax leaves them, would otherwise send
+// whole passes the long way (25M, K = 8, one gradient in a hundred times 1e-22:
+// 1114 us with a bound on a alone, 424 with CUDA's functions throughout, 245 so,
+// as without such gradients).  NaN fails.  One add-and-compare instruction per
+// bound, and no branch among the pushes: a pass looks once, at its end, and forms
 // the quads that left the range again (exact_quad).
 template <int ARITH> struct Guard {
     __device__ __forceinline__ bool ok() const { return true; }
@@ -185,6 +191,10 @@ __device__ __forceinline__ Pair minus_quotient2(Pair a, Pair v, Pair minus_z) {
     return fma2(fma2(v, minus_q, a), minus_z, minus_q);
 }
 
+// The scaled quotient's lowest value in range is 2^-26, theta's 2^-40: the weight
+// that brings both to one line.
+constexpr float kQuotientScale = 1099511627776.0f, kThetaWeight = 16384.0f;   // 2^40, 2^14
+
 // fasgd_update_exact on two parameters, the same bits.  25M, K = 8 / 16, push +
 // apply + pull: 464 us with CUDA's functions (K = 8), 282 / 517 with the negations
 // as operations of their own, 273 / 494 now.
@@ -209,10 +219,15 @@ __device__ __forceinline__ void exact_update2(Pair& theta, Pair& n, Pair& b, Pai
     v = add2(product2(pair(sp.beta, sp.beta), v, sp), step);
     unpack(v, x, y);
     guard.see_v(x, y);
-    const Pair a = mul2(pair(coef, coef), g);
-    unpack(a, x, y);
-    guard.see_a(x, y);
-    theta = add2(theta, minus_quotient2(a, v, minus_reciprocal2(v)));
+    // a and q come times 2^40 (exact where a is normal), so that a small a leaves
+    // no subnormal residual; the last operation scales q back and rounds once.
+    const float up = coef * kQuotientScale;
+    const Pair minus_q = minus_quotient2(mul2(pair(up, up), g), v, minus_reciprocal2(v));
+    float tx, ty;
+    unpack(minus_q, x, y);
+    unpack(mul2(theta, pair(kThetaWeight, kThetaWeight)), tx, ty);
+    guard.see_q(x, y, tx, ty);
+    theta = fma2(minus_q, pair(1.f / kQuotientScale, 1.f / kQuotientScale), theta);
 }
 
 // Arithmetic of a pass: hardware approximations (subnormal-preserving or
@@ -220,7 +235,7 @@ __device__ __forceinline__ void exact_update2(Pair& theta, Pair& n, Pair& b, Pai
 enum : int { kArithApprox = 0, kArithApproxFtz = 1, kArithExact = 2 };
 
 template <> struct Guard<kArithExact> {
-    uint32_t rad = 0, v = 0, a_min = 0xffffffffu, a_max = 0;
+    uint32_t rad = 0, v = 0, q_min = 0xffffffffu, q_max = 0;
     __device__ __forceinline__ void see_rad(float x, float y) {
         rad = __viaddmax_u32(__float_as_uint(x), 0u - kRadLo, rad);
         rad = __viaddmax_u32(__float_as_uint(y), 0u - kRadLo, rad);
@@ -229,17 +244,24 @@ template <> struct Guard<kArithExact> {
         v = __viaddmax_u32(__float_as_uint(x), 0u - kLo, v);
         v = __viaddmax_u32(__float_as_uint(y), 0u - kLo, v);
     }
-    __device__ __forceinline__ void see_a(float x, float y) {
-        const uint32_t mx = __float_as_uint(x) & 0x7fffffffu, my = __float_as_uint(y) & 0x7fffffffu;
-        a_min = __viaddmin_u32(mx, 0xffffffffu, a_min);   // a zero wraps to the largest
-        a_min = __viaddmin_u32(my, 0xffffffffu, a_min);
-        a_max = max(a_max, max(mx, my));
+    // The larger of the scaled quotient and the weighted theta, NaN from either.
+    static __device__ __forceinline__ uint32_t larger(float q, float t) {
+        float m;
+        asm("max.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(fabsf(q)), "f"(fabsf(t)));
+        return __float_as_uint(m);
+    }
+    __device__ __forceinline__ void see_q(float x, float y, float tx, float ty) {
+        const uint32_t mx = larger(x, tx), my = larger(y, ty);
+        q_min = __viaddmin_u32(mx, 0xffffffffu, q_min);   // zeros wrap to the largest
+        q_min = __viaddmin_u32(my, 0xffffffffu, q_min);
+        q_max = max(q_max, max(mx, my));
     }
     __device__ __forceinline__ bool ok() const {
-        return rad <= kRadHi - kRadLo && v <= kHi - kLo && a_min >= kLo - 1 && a_max <= kHi;
+        return rad <= kRadHi - kRadLo && v <= kHi - kLo && q_min >= kQLo - 1 && q_max <= kQHi;
     }
     static constexpr uint32_t kRadLo = 27u << 23, kRadHi = 227u << 23;   // 2^-100, 2^100
     static constexpr uint32_t kLo = 67u << 23, kHi = 187u << 23;         // 2^-60, 2^60
+    static constexpr uint32_t kQLo = 101u << 23, kQHi = 247u << 23;      // 2^-26, 2^120 (times 2^40)
 };
 
 template <int ARITH, bool STD>
@@ -293,21 +315,22 @@ template <bool STD>
 __device__ __noinline__ QuadState exact_quad(const float* theta, const float* n, const float* b,
                                              const float* v, const float* g0, const float* const* grad,
                                              const float* coef, int K, int64_t e, const StatParams& sp) {
-    float o[4][4];
-    for (int i = 0; i < 4; ++i) {
-        float th = theta[e + i], x = n[e + i], y = b[e + i], z = v[e + i];
-        for (int k = 0; k < K; ++k)
-            fasgd_update_exact<STD>(th, x, y, z, (k == 0 ? g0 : grad[k])[e + i], coef[k], sp);
-        o[0][i] = th;
-        o[1][i] = x;
-        o[2][i] = y;
-        o[3][i] = z;
-    }
     QuadState q;
-    q.th = make_float4(o[0][0], o[0][1], o[0][2], o[0][3]);
-    q.n = make_float4(o[1][0], o[1][1], o[1][2], o[1][3]);
-    q.b = make_float4(o[2][0], o[2][1], o[2][2], o[2][3]);
-    q.v = make_float4(o[3][0], o[3][1], o[3][2], o[3][3]);
+    q.th = *reinterpret_cast<const float4*>(theta + e);
+    q.n = *reinterpret_cast<const float4*>(n + e);
+    q.b = *reinterpret_cast<const float4*>(b + e);
+    q.v = *reinterpret_cast<const float4*>(v + e);
+    float4 g = *reinterpret_cast<const float4*>(g0 + e);
+#pragma unroll 1
+    for (int k = 0; k < K; ++k) {
+        float4 next = g;
+        if (k + 1 < K) next = *reinterpret_cast<const float4*>(grad[k + 1] + e);
+        fasgd_update_exact<STD>(q.th.x, q.n.x, q.b.x, q.v.x, g.x, coef[k], sp);
+        fasgd_update_exact<STD>(q.th.y, q.n.y, q.b.y, q.v.y, g.y, coef[k], sp);
+        fasgd_update_exact<STD>(q.th.z, q.n.z, q.b.z, q.v.z, g.z, coef[k], sp);
+        fasgd_update_exact<STD>(q.th.w, q.n.w, q.b.w, q.v.w, g.w, coef[k], sp);
+        g = next;
+    }
     return q;
 }
 

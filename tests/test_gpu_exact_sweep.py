@@ -2,7 +2,8 @@
 (update.cuh) against CUDA's correctly rounded functions, bit for bit: root and
 reciprocal for every fp32 value of the range in which the passes use them
 (2^-100 to 2^100 under the root, 2^-60 to 2^60 for the reciprocal), the quotient
-on pairs where a rounding can go wrong.  The kernels are compiled here, from the
+on pairs where a rounding can go wrong (the passes scale the dividend by 2^40 and
+use quotients from 2^-26 to 2^120).  The kernels are compiled here, from the
 header that the passes are compiled from."""
 
 import subprocess
@@ -76,6 +77,13 @@ __global__ void sweep(int kind, uint64_t from, uint64_t n, Result* r) {
             quotient(r, __uint_as_float(__float_as_uint(in_range((uint32_t)h, random_exponent(h))) | sign),
                      in_range((uint32_t)g, random_exponent(g)), in_range((uint32_t)(h >> 23), random_exponent(g) >> 9),
                      in_range((uint32_t)(g >> 23), random_exponent(h) >> 9));
+        } else if (kind == 5) {   // all exponents: of v, and of a for quotients from 2^-25 to 2^118
+            const uint32_t ev = 67u + random_exponent(h) % 120u, eq = 102u + random_exponent(g) % 144u;
+            const int ea = (int)eq + (int)ev - 127;
+            if (ea < 1 || ea > 253) continue;
+            const float a = __uint_as_float(((uint32_t)g & 0x7fffffu) | ((uint32_t)ea << 23) | sign);
+            const float v = __uint_as_float(((uint32_t)h & 0x7fffffu) | (ev << 23));
+            quotient(r, a, a, v, v);
         } else if (kind == 3) {
             // v in [1, 2), q in [1, 2) with a 25th bit set: a is the float next to
             // q v, so that a / v is as near to a midpoint as it gets; times powers of two.
@@ -129,7 +137,7 @@ def program(tmp_path_factory):
 BITS = 1 << 23
 SWEEPS = {"root": (0, 27 * BITS, 200 * BITS + 1), "reciprocal": (1, 67 * BITS, 120 * BITS + 1),
           "quotient random": (2, 12345, 1 << 34), "quotient near midpoints": (3, 999, 1 << 32),
-          "quotient mantissas at the ends": (4, 0, 1024 * BITS), "quotient edges": (-1, 0, 0)}
+          "quotient mantissas at the ends": (4, 0, 1024 * BITS), "quotient all exponents": (5, 777, 1 << 32), "quotient edges": (-1, 0, 0)}
 
 
 @pytest.mark.parametrize("name", SWEEPS)
