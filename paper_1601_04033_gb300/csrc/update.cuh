@@ -139,13 +139,13 @@ __device__ __forceinline__ Pair product2(Pair a, Pair b, const StatParams& sp) {
 // What the pushes of a pass saw, kept while they are applied: whether the
 // chains of exact_update2 gave the correctly rounded sequence throughout.  That
 // holds for rad in [2^-100, 2^100], v in [2^-60, 2^60] and a quotient q = a / v,
-// a = fl(coef g), that is zero or of magnitude in [2^-66, 2^80]: a and q are then
+// a = fl(coef g), that is zero or of magnitude in [2^-66, 2^94]: a and q are then
 // normal, no intermediate is subnormal and no residual rounded.  A smaller q does
 // no harm either where |theta| is 2^-40 or more: half the gap to its neighbours is
 // at least 2^-65, so theta stays as it is whatever q rounds to.  Gradients far
 // below their neighbours, as a saturated softmax leaves them, would otherwise send
 // whole passes the long way (25M, K = 8, one gradient in a hundred times 1e-22:
-// 1114 us with a bound on a alone, 424 with CUDA's functions throughout, 245 so,
+// 1114 us with a bound on a alone, 424 with CUDA's functions throughout, 247 so,
 // as without such gradients).  NaN fails.  One add-and-compare instruction per
 // bound, and no branch among the pushes: a pass looks once, at its end, and forms
 // the quads that left the range again (exact_quad).
@@ -191,9 +191,8 @@ __device__ __forceinline__ Pair minus_quotient2(Pair a, Pair v, Pair minus_z) {
     return fma2(fma2(v, minus_q, a), minus_z, minus_q);
 }
 
-// The scaled quotient's lowest value in range is 2^-26, theta's 2^-40: the weight
-// that brings both to one line.
-constexpr float kQuotientScale = 1099511627776.0f, kThetaWeight = 16384.0f;   // 2^40, 2^14
+// Brings the lowest quotient in range, 2^-66, to theta's line, 2^-40.
+constexpr float kQuotientScale = 67108864.0f;   // 2^26
 
 // fasgd_update_exact on two parameters, the same bits.  25M, K = 8 / 16, push +
 // apply + pull: 464 us with CUDA's functions (K = 8), 282 / 517 with the negations
@@ -219,13 +218,14 @@ __device__ __forceinline__ void exact_update2(Pair& theta, Pair& n, Pair& b, Pai
     v = add2(product2(pair(sp.beta, sp.beta), v, sp), step);
     unpack(v, x, y);
     guard.see_v(x, y);
-    // a and q come times 2^40 (exact where a is normal), so that a small a leaves
-    // no subnormal residual; the last operation scales q back and rounds once.
+    // a and q come times 2^26 (exact where a is normal): a small a then leaves no
+    // rounded residual (its last bit is 2^-146 or more), and one comparison serves
+    // q and theta.  The last operation scales q back and rounds once.
     const float up = coef * kQuotientScale;
     const Pair minus_q = minus_quotient2(mul2(pair(up, up), g), v, minus_reciprocal2(v));
     float tx, ty;
     unpack(minus_q, x, y);
-    unpack(mul2(theta, pair(kThetaWeight, kThetaWeight)), tx, ty);
+    unpack(theta, tx, ty);
     guard.see_q(x, y, tx, ty);
     theta = fma2(minus_q, pair(1.f / kQuotientScale, 1.f / kQuotientScale), theta);
 }
@@ -244,7 +244,7 @@ template <> struct Guard<kArithExact> {
         v = __viaddmax_u32(__float_as_uint(x), 0u - kLo, v);
         v = __viaddmax_u32(__float_as_uint(y), 0u - kLo, v);
     }
-    // The larger of the scaled quotient and the weighted theta, NaN from either.
+    // The larger of the scaled quotient and theta, NaN from either.
     static __device__ __forceinline__ uint32_t larger(float q, float t) {
         float m;
         asm("max.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(fabsf(q)), "f"(fabsf(t)));
@@ -261,7 +261,7 @@ template <> struct Guard<kArithExact> {
     }
     static constexpr uint32_t kRadLo = 27u << 23, kRadHi = 227u << 23;   // 2^-100, 2^100
     static constexpr uint32_t kLo = 67u << 23, kHi = 187u << 23;         // 2^-60, 2^60
-    static constexpr uint32_t kQLo = 101u << 23, kQHi = 247u << 23;      // 2^-26, 2^120 (times 2^40)
+    static constexpr uint32_t kQLo = 87u << 23, kQHi = 247u << 23;       // 2^-40, 2^120
 };
 
 template <int ARITH, bool STD>

@@ -77,7 +77,7 @@ def test_exact_mode_on_steps_far_below_theta(variant, eps, budget):
     P = 400_003
     line = np.float32(2.0 ** -40)
     edge = np.float32([line, np.nextafter(line, np.float32(0)), -line, 0.0, -0.0, 1e-45, -1e-40, 2.0 ** -66,
-                       2.0 ** -41, 2.0 ** -39, 1.0, 2.0 ** 105, 2.0 ** 106])
+                       2.0 ** -41, 2.0 ** -39, 1.0, 2.0 ** 119, 2.0 ** 121])
     theta = np.where(rng.random(P) < 0.5, np.resize(edge, P), _wild(rng, P, -149, 10)).astype(np.float32)
     # Large n leaves v to its old value, so quotients spread over all exponents.
     n = np.where(rng.random(P) < 0.7, _wild(rng, P, 80, 99, False), _wild(rng, P, -30, 0, False)).astype(np.float32)

@@ -2,8 +2,8 @@
 (update.cuh) against CUDA's correctly rounded functions, bit for bit: root and
 reciprocal for every fp32 value of the range in which the passes use them
 (2^-100 to 2^100 under the root, 2^-60 to 2^60 for the reciprocal), the quotient
-on pairs where a rounding can go wrong (the passes scale the dividend by 2^40 and
-use quotients from 2^-26 to 2^120).  The kernels are compiled here, from the
+on pairs where a rounding can go wrong (the passes scale the dividend by 2^26 and
+use quotients from 2^-40 to 2^120).  The kernels are compiled here, from the
 header that the passes are compiled from."""
 
 import subprocess
@@ -77,8 +77,8 @@ __global__ void sweep(int kind, uint64_t from, uint64_t n, Result* r) {
             quotient(r, __uint_as_float(__float_as_uint(in_range((uint32_t)h, random_exponent(h))) | sign),
                      in_range((uint32_t)g, random_exponent(g)), in_range((uint32_t)(h >> 23), random_exponent(g) >> 9),
                      in_range((uint32_t)(g >> 23), random_exponent(h) >> 9));
-        } else if (kind == 5) {   // all exponents: of v, and of a for quotients from 2^-25 to 2^118
-            const uint32_t ev = 67u + random_exponent(h) % 120u, eq = 102u + random_exponent(g) % 144u;
+        } else if (kind == 5) {   // all exponents: of v, and of a for quotients from 2^-39 to 2^118
+            const uint32_t ev = 67u + random_exponent(h) % 120u, eq = 88u + random_exponent(g) % 158u;
             const int ea = (int)eq + (int)ev - 127;
             if (ea < 1 || ea > 253) continue;
             const float a = __uint_as_float(((uint32_t)g & 0x7fffffu) | ((uint32_t)ea << 23) | sign);
