@@ -469,6 +469,7 @@ cudaError_t launch_rule(const DenseArgs& a, int num_sms, cudaStream_t stream) {
     //          8: 253 -> 254         12: 316 -> 312    16: 375 (same)   32: 631 -> 601
     //   exact  3: 204 -> 190         4: 223 -> 207     5: 222 (same)
     //          6: 238 -> 232         7: 260 -> 247     8: 273     16: 494
+    //          (with the present guard of the quotient 5: 221, 6: 232, 7: 257, 16: 491)
     //   SGD    K = 3: 103 -> 102     5: 133.4 -> 131.6 6: 148 -> 146     8: 182 -> 174
     //          12: 242 -> 232        16: 300 -> 287    32: 531 -> 512
     //
